@@ -188,20 +188,23 @@ __device__ __forceinline__ void collide_increment(const float (&f)[9], float rr,
 }
 
 // Store of the post-collision, recoloured populations of one node (Eq.
-// eq_re_color) in the FP32 layout float[18][nodes] at `out` (the node's
-// address in plane 0).  The minority colour is formed directly and the
+// eq_re_color) in the FP32 layout float[18][nodes]: column x of the lattice
+// row at `row` in plane 0 (a value common to the CTA, so that the eighteen
+// plane addresses are too).  The minority colour is formed directly and the
 // majority as the rest of f+, so that R++ + B++ = f+ holds to one rounding of
 // the majority.  (sx, sy) is the red segregation vector
 // beta phi rho_R rho_B / rho e.
-__device__ __forceinline__ void store_recoloured_f32(float* out, size_t nodes, const float (&fp)[9], float rr,
-                                                     float rb, float inv_rho, float sx, float sy) {
+__device__ __forceinline__ void store_recoloured_f32(float* row, unsigned x, size_t nodes, const float (&fp)[9],
+                                                     float rr, float rb, float inv_rho, float sx, float sy) {
     const bool red_major = rr >= rb;
     const float amin = (red_major ? rb : rr) * inv_rho;
     const float smin = red_major ? -1.0f : 1.0f;  // minority's sign of the segregation term
     float seg[9];
     segregation(smin * sx, smin * sy, seg);
-    float* out_min = out + (red_major ? 9 * nodes : 0);
-    float* out_maj = out + (red_major ? 0 : 9 * nodes);
+    auto put = [&](int i, float cmin, float cmaj) {
+        __stcs(row + static_cast<size_t>(i) * nodes + x, red_major ? cmaj : cmin);
+        __stcs(row + static_cast<size_t>(9 + i) * nodes + x, red_major ? cmin : cmaj);
+    };
     // links in pairs as packed FP32x2 FMAs (fp - cmin as cmin * -1 + fp: the
     // same single rounding as the subtraction)
     const float2 a2 = make_float2(amin, amin), m1 = make_float2(-1.0f, -1.0f);
@@ -210,14 +213,11 @@ __device__ __forceinline__ void store_recoloured_f32(float* out, size_t nodes, c
         const float2 f2 = make_float2(fp[i], fp[i + 1]);
         const float2 cmin = __ffma2_rn(a2, f2, make_float2(seg[i], seg[i + 1]));
         const float2 cmaj = __ffma2_rn(cmin, m1, f2);
-        __stcs(out_min + i * nodes, cmin.x);
-        __stcs(out_min + (i + 1) * nodes, cmin.y);
-        __stcs(out_maj + i * nodes, cmaj.x);
-        __stcs(out_maj + (i + 1) * nodes, cmaj.y);
+        put(i, cmin.x, cmaj.x);
+        put(i + 1, cmin.y, cmaj.y);
     }
     const float cmin8 = fmaf(amin, fp[8], seg[8]);
-    __stcs(out_min + 8 * nodes, cmin8);
-    __stcs(out_maj + 8 * nodes, fp[8] - cmin8);
+    put(8, cmin8, fp[8] - cmin8);
 }
 
 }  // namespace cmrt

@@ -1265,7 +1265,7 @@ __global__ void __launch_bounds__(kAT) k_step_planes(const float* __restrict__ p
     const float inv = (mag2 >= kNormalTau * kNormalTau) ? rsqrtf(mag2) : 0.0f;
     const float phim = fmaf(P.kphi_r, rr, P.kphi_b * rb) * inv_rho;
     const float sg = P.beta * (rr * rb) * inv_rho * phim * inv;
-    store_recoloured_f32(dst + o, L.n, fp, rr, rb, inv_rho, sg * gx, sg * gy);
+    store_recoloured_f32(dst + L.row[reach<ORDER>()], x, L.n, fp, rr, rb, inv_rho, sg * gx, sg * gy);
 }
 
 __global__ void __launch_bounds__(kAT) k_fields_planes(const StepParams P, const float* __restrict__ S,

@@ -38,6 +38,8 @@
 // reconstruction M^{-1} dm is grouped by the parity of each column k^(p)
 // under c -> -c, which the k vectors of App. A have by construction.
 #include <atomic>
+#include <cmath>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -200,7 +202,7 @@ struct LayoutF32 {
     __device__ __forceinline__ static void store(char* dst, size_t nodes, size_t node, const float (&fp)[9],
                                                  float rr, float rb, float inv_rho, float sx, float sy, float,
                                                  float, const StepParams&) {
-        store_recoloured_f32(reinterpret_cast<float*>(dst) + node, nodes, fp, rr, rb, inv_rho, sx, sy);
+        store_recoloured_f32(reinterpret_cast<float*>(dst) + node, 0u, nodes, fp, rr, rb, inv_rho, sx, sy);
     }
 };
 
@@ -896,12 +898,399 @@ __device__ __forceinline__ void chain_tile(const Rings<L, WALLS>& R, const unsig
     }
 }
 
+
+// Local kinematic viscosity (Sec. 2: nu(rho^N) = (2 / lambda_3 - 1) / 6), rho^N by Eq. equ_rhoN_def.
+__device__ __forceinline__ float node_viscosity(float rr, float rb, float inv_rho, const StepParams& P) {
+    if (P.visc_mode != 0) return P.eta * inv_rho;
+    const float ra = rr * P.inv_rho0_r, ba = rb * P.inv_rho0_b;
+    const float rn = (ra - ba) * rcp(ra + ba);
+    return fmaf(0.5f * (P.nu_r - P.nu_b), rn, 0.5f * (P.nu_r + P.nu_b));
+}
+
+// ---------------------------------------------------------------------------
+// The march: the row pipeline of one tile with FP32 storage.
+//
+// A CTA of 128 threads, one per window column, runs all four stages of every
+// row itself; four such CTAs (16 warps) share an SM.  Row iteration k
+// (r = y0 - 3 + k) runs, with one barrier before each group,
+//   D (row r - 4), A (row r) | B (row r - 1) | C (row r - 2).
+// What bounds it: HBM.  144 B per node are the algorithm's; to stream them an
+// SM has to keep 40 KB in flight and to issue few instructions per node, and
+// both come from where the data between the stages lives:
+// - Every population is gathered exactly once, by stage A.  A slot of shared
+//   memory holds what gather row r needs (plane q from row r - c_y(q)), so a
+//   row is dead as soon as A has read it and three slots (one in use, two in
+//   flight) serve where a ring of whole rows kept for stage D needed nine.
+// - Stage D gets f, rho_R and rho_B of its row from registers, where A left
+//   them four iterations before (f[4][9] and so on below, the slot a
+//   compile-time constant in a loop unrolled four times), instead of
+//   gathering and summing the eighteen populations again.
+// - The smaller shared memory (42 KB against 114 KB) lets four CTAs of four
+//   warps stand on an SM, 512 columns in flight against 256 of the
+//   warp-specialised form that 16-bit storage keeps (chain_tile), each with
+//   the whole work of a row to overlap the others' barriers.
+// - Instructions per node fell from 836 to 596.
+// Measured at 8192^2 (drops, FP32): 1982 us per step before (33.9 GLUPS,
+// 4.9 TB/s), 1646 us now (40.8 GLUPS, 5.9 TB/s, 87 % of the measured copy);
+// 2048^2 143 -> 122 us.  Two and four slots: 1851 and 1678 us.  Three CTAs
+// per SM (168 registers): 1698 us.  256-column windows (two CTAs of eight
+// warps) 1930 us: fewer barrier domains to overlap.
+// ---------------------------------------------------------------------------
+constexpr int kMarchCtas = 4;   // resident CTAs (of 128 threads) per SM
+constexpr int kMarchSlots = 3;  // population rows in shared memory: one in use, two in flight
+constexpr int kMarchRows = 28;  // stage rings, four rows each: chi_R, chi_B, Phi', n-hat x, y, u x, y
+constexpr int kMarchPop = kPlanes * kWin;  // floats of a population slot
+constexpr int kMarchBytes = 4 * (kMarchSlots * kMarchPop + kMarchRows * kWin);
+static_assert(kMarchCtas * (kMarchBytes + 1024) <= 228 * 1024, "resident march CTAs");
+
+template <int C>
+using Const = std::integral_constant<int, C>;
+
+// This thread's share of the copy of a gather row: with VEC (nx a multiple of
+// 4) 16-byte chunks, warp w copying planes w, w + 4, ... and a lane four
+// columns; otherwise its own column of every plane.  PRE: the populations
+// already lie where they are needed (the public layout).
+template <bool VEC, bool WALLS, bool PRE>
+struct MarchCopy {
+    static constexpr int kN = VEC ? (kPlanes + 3) / 4 : 1;
+    const char* ptr[kN];  // column of plane q in row -c_y(q)
+    size_t row_bytes, plane_bytes;
+    int ny;
+    unsigned soff;
+    __device__ __forceinline__ static int plane_of(int m) { return static_cast<int>(threadIdx.x >> 5) + 4 * m; }
+    // c_y of the link of plane q
+    __device__ __forceinline__ static int plane_cy(int q) {
+        const int l = q >= 9 ? q - 9 : q;
+        return PRE ? 0 : (l >= 5 && l <= 7 ? -1 : (l >= 1 && l <= 3 ? 1 : 0));
+    }
+    __device__ __forceinline__ void init(const char* state, int x0, int nx, int ny_) {
+        ny = ny_;
+        row_bytes = static_cast<size_t>(nx) * 4;
+        plane_bytes = row_bytes * ny;
+        soff = VEC ? threadIdx.x * 16 : threadIdx.x * 4;
+        if (VEC) {
+            const int col = wrap(x0 - kHalo + static_cast<int>(threadIdx.x & 31) * 4, nx);
+#pragma unroll
+            for (int m = 0; m < kN; ++m)
+                ptr[m] = state + plane_bytes * plane_of(m) + static_cast<size_t>(col) * 4 -
+                         static_cast<ptrdiff_t>(row_bytes) * plane_cy(plane_of(m));
+        } else {
+            ptr[0] = state + static_cast<size_t>(wrap(x0 - kHalo + static_cast<int>(threadIdx.x), nx)) * 4;
+        }
+    }
+    __device__ __forceinline__ int wrap_row(int r) const { return WALLS || (r >= 0 && r < ny) ? r : wrap(r, ny); }
+    // byte offset from plane q's row -c_y(q) to the row that gather row r takes from it
+    __device__ __forceinline__ ptrdiff_t row_off(int r, int q, int cy) const {
+        int g = r - cy;
+        if (WALLS) {
+            // half-way bounce-back: the node's own row of the opposite link's plane
+            if (g < 0 || g >= ny) return static_cast<ptrdiff_t>(plane_bytes) * (cy > 0 ? 4 : -4) +
+                                         static_cast<ptrdiff_t>(row_bytes) * (r + cy);
+        } else if (g < 0 || g >= ny) {
+            g = wrap(g, ny);
+        }
+        return static_cast<ptrdiff_t>(row_bytes) * (g + cy);
+    }
+    // the populations of gather row r into a slot: plane q from row r - c_y(q)
+    __device__ __forceinline__ void issue(unsigned slot_addr, int r) const {
+        const unsigned d = slot_addr + soff;
+        const bool inner = r >= 1 && r <= ny - 2;
+        if (VEC) {
+            if (inner) {
+                const ptrdiff_t o = static_cast<ptrdiff_t>(row_bytes) * r;
+#pragma unroll
+                for (int m = 0; m < kN; ++m)
+                    if (4 * m + 3 < kPlanes || plane_of(m) < kPlanes) cp_async16(d + m * 16 * kThreads, ptr[m] + o);
+            } else {
+#pragma unroll
+                for (int m = 0; m < kN; ++m) {
+                    const int q = plane_of(m);
+                    if (q < kPlanes) cp_async16(d + m * 16 * kThreads, ptr[m] + row_off(r, q, plane_cy(q)));
+                }
+            }
+        } else {
+            // source rows of the planes with c_y = -1, 0, 1 (bytes from the same plane's row 0)
+            const ptrdiff_t om = PRE ? 0 : row_off(r, 5, -1) + static_cast<ptrdiff_t>(row_bytes);
+            const ptrdiff_t oz = static_cast<ptrdiff_t>(row_bytes) * wrap_row(r);
+            const ptrdiff_t op = PRE ? 0 : row_off(r, 1, 1) - static_cast<ptrdiff_t>(row_bytes);
+#pragma unroll
+            for (int q = 0; q < kPlanes; ++q) {
+                const int cy = PRE ? 0 : lcy(q % 9);
+                cp_async4(d + q * kWin * 4, ptr[0] + (static_cast<ptrdiff_t>(plane_bytes) * q + (cy > 0 ? op : (cy < 0 ? om : oz))));
+            }
+        }
+    }
+};
+
+// The strip [x0, x0 + 120) of rows [y0, y0 + rows).  Window columns whose
+// neighbours lie outside the window hold garbage, one more on each side after
+// every stage; the four halo columns keep it off the owned ones.  Leaves no
+// copy in flight.
+//
+// Ring slots: row r - j of the iteration is in slot (k - j) mod 4 of every
+// stage ring.  chi is read down to row r - 2 by B, n-hat to r - 3 by C (and
+// r - 4 by D, the own column), u and Phi' to r - 5 by D, each at least one
+// barrier before its slot is written again.  Beyond a wall a stage writes the
+// mirrored row together with the wall row, into the slot of the row four
+// away, which no later stage reads any more.
+template <bool VEC, bool WALLS, Pass MODE, bool PRE>
+__device__ __forceinline__ void march_tile(float* __restrict__ smem, const char* __restrict__ src,
+                                           char* __restrict__ dst, const StepParams& P, const int x0, const int y0,
+                                           const int rows, const FieldOut& fo, unsigned* __restrict__ flag,
+                                           DiagAcc& acc) {
+    constexpr bool kStep = MODE == Pass::Step || MODE == Pass::StepFields;
+    const int t = static_cast<int>(threadIdx.x);
+    const int nx = P.nx, ny = P.ny;
+    const size_t nodes = static_cast<size_t>(nx) * ny;
+    const int y_end = min(y0 + rows, ny);
+    const int r_first = y0 - 3;
+    const int r_last = y_end + 2;  // last gathered row
+    const int iters = (y_end - y0) + 7;
+    const unsigned pop_addr = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+    float* ring = smem + kMarchSlots * kMarchPop + t;  // this thread's column of the stage rings
+    auto row_ok = [&](int r) { return !WALLS || (r >= 0 && r < ny); };
+    const int gx_own = x0 + t - kHalo;
+    const bool own_col = t >= kHalo && t < kWin - kHalo && gx_own < nx;
+    auto owned = [&](int r) { return MODE == Pass::StepFields && own_col && r >= y0 && r < y_end; };
+    auto fwd = [&](int plane, int r) -> float& {
+        return fo.fwd[static_cast<size_t>(plane) * nodes + static_cast<size_t>(r) * nx + gx_own];
+    };
+    // ring rows (column t): field f of the row in slot c
+    auto R = [&](int f, int c) { return ring + (f * 4 + c) * kWin; };
+    constexpr int kChiR = 0, kChiB = 1, kPhi = 2, kNx = 3, kNy = 4, kUx = 5, kUy = 6;
+    auto dx = [&](int f, int n, int m, int s) {
+        const float *a = R(f, n), *b = R(f, m), *c = R(f, s);
+        return ddx(b[1], b[-1], a[1], a[-1], c[1], c[-1]);
+    };
+    auto dy = [&](int f, int n, int s) {
+        const float *a = R(f, n), *c = R(f, s);
+        return ddy(a[0], c[0], a[1], a[-1], c[1], c[-1]);
+    };
+
+    MarchCopy<VEC, WALLS, PRE> copy;
+    copy.init(src, x0, nx, ny);
+    auto issue = [&](int r, int slot) {
+        if (r <= r_last && row_ok(r)) copy.issue(pop_addr + static_cast<unsigned>(slot * kMarchPop * 4), r);
+        cp_commit();
+    };
+#pragma unroll
+    for (int j = 0; j < kMarchSlots - 1; ++j) issue(r_first + j, j);
+
+    // what the later stages of this column need, slot = row iteration mod 4
+    float f[4][9], rr[4], rb[4], jx[4], jy[4], gx[4], gy[4], Gx[4], Gy[4];
+
+    auto iteration = [&](auto C, const int k) {
+        constexpr int c0 = decltype(C)::value;                    // slot of row r
+        constexpr int c1 = (c0 + 3) & 3, c2 = (c0 + 2) & 3, c3 = (c0 + 1) & 3;  // of rows r - 1, r - 2, r - 3
+        const int r = r_first + k;
+        cp_wait<kMarchSlots - 2>();
+        __syncthreads();
+        // row r + 2 goes to the slot that row r - 1 left
+        issue(r + kMarchSlots - 1, (k + kMarchSlots - 1) % kMarchSlots);
+        // ---- D: row r - 4 (FIFO slot c0): rows r - 3, r - 4, r - 5 of the rings in slots c3, c0, c1
+        const int yd = r - 4;
+        if (yd >= y0 && yd < y_end && own_col) {
+            const float drr = rr[c0], drb = rb[c0];
+            const float rho = drr + drb;
+            const float ux = R(kUx, c0)[0], uy = R(kUy, c0)[0];
+            if (kStep) {
+                if (!isfinite(rho)) atomicOr(flag, 1u);
+                const float dPx = dx(kPhi, c3, c0, c1), dPy = dy(kPhi, c3, c1);
+                const float divu = dx(kUx, c3, c0, c1) + dy(kUy, c3, c1);
+                const float inv_rho = rcp(rho);
+                const float nu = node_viscosity(drr, drb, inv_rho, P);
+                float fp[9];
+                collide_increment(f[c0], drr, drb, rho, nu, ux, uy, Gx[c0], Gy[c0], dPx, dPy, divu, P, fp);
+                const float ex = -R(kNx, c0)[0];
+                const float ey = -R(kNy, c0)[0];
+                const float phim = fmaf(P.kphi_r, drr, P.kphi_b * drb) * inv_rho;
+                const float sg = P.beta * (drr * drb) * inv_rho * phim;
+                store_recoloured_f32(reinterpret_cast<float*>(dst) + static_cast<size_t>(yd) * nx, gx_own, nodes, fp,
+                                     drr, drb, inv_rho, sg * ex, sg * ey);
+            } else if (MODE == Pass::Fields) {
+                const size_t o = static_cast<size_t>(yd) * nx + gx_own;
+                if (fo.rho_r) fo.rho_r[o] = drr;
+                if (fo.rho_b) fo.rho_b[o] = drb;
+                if (fo.ux) fo.ux[o] = ux;
+                if (fo.uy) fo.uy[o] = uy;
+                if (fo.p) fo.p[o] = fmaf(P.cs2_r, drr, P.cs2_b * drb);
+            } else {
+                const float* F = f[c0];
+                const float mx = (F[1] + F[7] + F[8]) - (F[3] + F[4] + F[5]);
+                const float my = (F[1] + F[2] + F[3]) - (F[5] + F[6] + F[7]);
+                if (isfinite(rho)) {
+                    acc.r += drr;
+                    acc.b += drb;
+                    acc.jx += mx;
+                    acc.jy += my;
+                    acc.u2 = fmax(acc.u2, static_cast<double>(ux) * ux + static_cast<double>(uy) * uy);
+                } else {
+                    acc.bad += 1.0;
+                }
+            }
+        }
+        // ---- A: moments of row r
+        if (r <= r_last && row_ok(r)) {
+            const float* slot = smem + (k % kMarchSlots) * kMarchPop + t;
+            const bool low = WALLS && r == 0, high = WALLS && r == ny - 1;
+            float fr[9], fb[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                // a link that comes from a wall: the slot holds the node's own reversed link
+                int d = PRE ? 0 : -lcx(i);
+                if (WALLS && !PRE && lcy(i) > 0 && low) d = 0;
+                if (WALLS && !PRE && lcy(i) < 0 && high) d = 0;
+                fr[i] = slot[i * kWin + d];
+                fb[i] = slot[(9 + i) * kWin + d];
+            }
+            const float2 rrb = sum9x2(fr, fb);
+            const float arr = rrb.x, arb = rrb.y;
+            const float ajx = ((fr[1] + fb[1]) + (fr[7] + fb[7])) + (fr[8] + fb[8]) -
+                              (((fr[3] + fb[3]) + (fr[5] + fb[5])) + (fr[4] + fb[4]));
+            const float ajy = ((fr[1] + fb[1]) + (fr[3] + fb[3])) + (fr[2] + fb[2]) -
+                              (((fr[5] + fb[5]) + (fr[7] + fb[7])) + (fr[6] + fb[6]));
+            const float a = arr * P.inv_rho0_r;
+            const float b = arb * P.inv_rho0_b;
+            const float inv_ab = rcp(__fadd_rn(a, b));
+            const float chr = a * inv_ab;
+            const float chb = b * inv_ab;
+            R(kChiR, c0)[0] = chr;
+            R(kChiB, c0)[0] = chb;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[c0][i] = fr[i] + fb[i];
+            rr[c0] = arr;
+            rb[c0] = arb;
+            jx[c0] = ajx;
+            jy[c0] = ajy;
+            if (owned(r)) {
+                fwd(kFwdRR, r) = arr;
+                fwd(kFwdRB, r) = arb;
+                fwd(kFwdCHR, r) = chr;
+                fwd(kFwdCHB, r) = chb;
+            }
+            if (WALLS && r == 0) {
+                R(kChiR, c1)[0] = chr;
+                R(kChiB, c1)[0] = chb;
+            }
+            if (WALLS && r == ny - 1) {
+                R(kChiR, c3)[0] = chr;
+                R(kChiB, c3)[0] = chb;
+            }
+        }
+        __syncthreads();
+        // ---- B: row r - 1
+        const int yb = r - 1;
+        if (yb >= y0 - 2 && yb <= y_end + 1 && row_ok(yb)) {
+            const bool use_b = R(kChiR, c1)[0] > 0.5f;
+            const float* base = ring + (use_b ? 4 * kWin : 0);
+            const float *n_ = base + c0 * kWin, *m_ = base + c1 * kWin, *s_ = base + c2 * kWin;
+            const float two = use_b ? -2.0f : 2.0f;
+            const float bgx = two * ddx(m_[1], m_[-1], n_[1], n_[-1], s_[1], s_[-1]);
+            const float bgy = two * ddy(n_[0], s_[0], n_[1], n_[-1], s_[1], s_[-1]);
+            const float mag2 = fmaf(bgx, bgx, bgy * bgy);
+            const float inv = (mag2 >= kNormalTau * kNormalTau) ? rsqrtf(mag2) : 0.0f;
+            const float nhx = -bgx * inv;
+            const float nhy = -bgy * inv;
+            gx[c1] = bgx;
+            gy[c1] = bgy;
+            R(kNx, c1)[0] = nhx;
+            R(kNy, c1)[0] = nhy;
+            if (owned(yb)) {
+                fwd(kFwdGX, yb) = bgx;
+                fwd(kFwdGY, yb) = bgy;
+            }
+            if (WALLS && yb == 0) {
+                R(kNx, c2)[0] = nhx;
+                R(kNy, c2)[0] = -nhy;
+            }
+            if (WALLS && yb == ny - 1) {
+                R(kNx, c0)[0] = nhx;
+                R(kNy, c0)[0] = -nhy;
+            }
+        }
+        __syncthreads();
+        // ---- C: row r - 2
+        const int yc = r - 2;
+        if (yc >= y0 - 1 && yc <= y_end && row_ok(yc)) {
+            const float K = P.curvature_mode == 0 ? dx(kNx, c1, c2, c3) + dy(kNy, c1, c3) : P.fixed_K;
+            const float rho = rr[c2] + rb[c2];
+            const float hk = P.half_sigma * K;
+            const float cGx = fmaf(hk, gx[c2], fmaf(rho, P.gacc_x, P.gvol_x));
+            const float cGy = fmaf(hk, gy[c2], fmaf(rho, P.gacc_y, P.gvol_y));
+            const float inv_rho = rcp(rho);
+            const float ux = fmaf(0.5f, cGx, jx[c2]) * inv_rho;
+            const float uy = fmaf(0.5f, cGy, jy[c2]) * inv_rho;
+            const float phip = fmaf(P.phip_r, rr[c2], P.phip_b * rb[c2]);
+            Gx[c2] = cGx;
+            Gy[c2] = cGy;
+            R(kUx, c2)[0] = ux;
+            R(kUy, c2)[0] = uy;
+            R(kPhi, c2)[0] = phip;
+            if (owned(yc)) {
+                fwd(kFwdPHIP, yc) = phip;
+                fwd(kFwdK, yc) = K;
+                fwd(kFwdGFX, yc) = cGx;
+                fwd(kFwdGFY, yc) = cGy;
+                fwd(kFwdUX, yc) = ux;
+                fwd(kFwdUY, yc) = uy;
+            }
+            if (WALLS && yc == 0) {
+                R(kUx, c3)[0] = -ux;
+                R(kUy, c3)[0] = -uy;
+                R(kPhi, c3)[0] = phip;
+            }
+            if (WALLS && yc == ny - 1) {
+                R(kUx, c1)[0] = -ux;
+                R(kUy, c1)[0] = -uy;
+                R(kPhi, c1)[0] = phip;
+            }
+        }
+    };
+    for (int k = 0; k < iters; k += 4) {
+        iteration(Const<0>{}, k);
+        if (k + 1 < iters) iteration(Const<1>{}, k + 1);
+        if (k + 2 < iters) iteration(Const<2>{}, k + 2);
+        if (k + 3 < iters) iteration(Const<3>{}, k + 3);
+    }
+    cp_wait<0>();
+}
+
 // A tile of rows [y0, y0 + rows) touches population rows y0 - 4 .. y0 + rows + 3
 // and runs its stages on rows y0 - 3 .. y0 + rows + 2.  When all of these lie
 // inside [1, ny - 2] no wall condition can apply (no bounce-back link, no
 // mirrored row is written or read), and the periodic form of the pipeline
 // computes exactly the same values with fewer instructions.
 __device__ __forceinline__ bool away_from_walls(int y0, int rows, int ny) { return y0 >= 5 && y0 + rows + 5 <= ny; }
+
+// The CTA's diagnostics: warp shuffles, then across the CTA's warps in shared memory (the rings are done).
+__device__ __forceinline__ void reduce_diag(const DiagAcc& acc, char* smem, double* __restrict__ partials) {
+    const int t = threadIdx.x;
+    double v[kDiagSlots] = {acc.r, acc.b, acc.jx, acc.jy, acc.u2, acc.bad};
+#pragma unroll
+    for (int j = 0; j < kDiagSlots; ++j) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const double o = __shfl_down_sync(0xffffffffu, v[j], off);
+            v[j] = (j == 4) ? fmax(v[j], o) : v[j] + o;
+        }
+    }
+    __syncthreads();
+    double* red = reinterpret_cast<double*>(smem);
+    const int warp = t >> 5, lane = t & 31;
+    if (lane == 0) {
+#pragma unroll
+        for (int j = 0; j < kDiagSlots; ++j) red[warp * kDiagSlots + j] = v[j];
+    }
+    __syncthreads();
+    if (t < kDiagSlots) {
+        double total = red[t];
+        for (int w = 1; w < kThreads / 32; ++w) {
+            const double o = red[w * kDiagSlots + t];
+            total = (t == 4) ? fmax(total, o) : total + o;
+        }
+        partials[(static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * kDiagSlots + t] = total;
+    }
+}
 
 template <class L, bool VEC, bool WALLS, Pass MODE, bool PRE>
 __global__ void __launch_bounds__(pass_threads(MODE), pass_ctas_per_sm<L>(MODE))
@@ -919,36 +1308,22 @@ __global__ void __launch_bounds__(pass_threads(MODE), pass_ctas_per_sm<L>(MODE))
     else
         chain_tile<L, VEC, WALLS, MODE, PRE>(make_rings<L, WALLS>(smem, P.ny), pop_addr, src, dst, P, x0, y0, rows, fo,
                                              flag, acc);
-    const int t = threadIdx.x;
+    if (MODE == Pass::Diag) reduce_diag(acc, smem, partials);
+}
 
-    if (MODE == Pass::Diag) {
-        // warp shuffle reduction, then across the CTA's warps in shared memory
-        double v[kDiagSlots] = {acc.r, acc.b, acc.jx, acc.jy, acc.u2, acc.bad};
-#pragma unroll
-        for (int j = 0; j < kDiagSlots; ++j) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const double o = __shfl_down_sync(0xffffffffu, v[j], off);
-                v[j] = (j == 4) ? fmax(v[j], o) : v[j] + o;
-            }
-        }
-        __syncthreads();
-        double* red = reinterpret_cast<double*>(smem);
-        const int warp = t >> 5, lane = t & 31;
-        if (lane == 0) {
-#pragma unroll
-            for (int j = 0; j < kDiagSlots; ++j) red[warp * kDiagSlots + j] = v[j];
-        }
-        __syncthreads();
-        if (t < kDiagSlots) {
-            double acc = red[t];
-            for (int w = 1; w < kThreads / 32; ++w) {
-                const double o = red[w * kDiagSlots + t];
-                acc = (t == 4) ? fmax(acc, o) : acc + o;
-            }
-            partials[(static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * kDiagSlots + t] = acc;
-        }
-    }
+template <bool VEC, bool WALLS, Pass MODE, bool PRE>
+__global__ void __launch_bounds__(kThreads, kMarchCtas)
+    k_march(const char* __restrict__ src, char* __restrict__ dst, const StepParams P, const int rows, FieldOut fo,
+            unsigned* __restrict__ flag, double* __restrict__ partials) {
+    pdl_begin();
+    extern __shared__ __align__(16) char smem[];
+    DiagAcc acc;
+    const int x0 = static_cast<int>(blockIdx.x) * kTileX, y0 = static_cast<int>(blockIdx.y) * rows;
+    if (WALLS && away_from_walls(y0, rows, P.ny))
+        march_tile<VEC, false, MODE, PRE>(reinterpret_cast<float*>(smem), src, dst, P, x0, y0, rows, fo, flag, acc);
+    else
+        march_tile<VEC, WALLS, MODE, PRE>(reinterpret_cast<float*>(smem), src, dst, P, x0, y0, rows, fo, flag, acc);
+    if (MODE == Pass::Diag) reduce_diag(acc, smem, partials);
 }
 
 // Batched ensemble: a persistent kernel over a work list of tiles of many
@@ -1078,13 +1453,41 @@ cudaError_t launch_layout(const void* src, void* dst, const StepParams& P, int r
     return launch_one<L, false, false, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
 }
 
+template <bool VEC, bool WALLS, Pass MODE, bool PRE>
+cudaError_t launch_march_one(const void* src, void* dst, const StepParams& P, int rows, FieldOut fo, unsigned* flag,
+                             double* partials, cudaStream_t s) {
+    static std::atomic<unsigned long long> configured{0};  // per device, set from any host thread
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(configured.load() & bit)) {
+        e = cudaFuncSetAttribute(k_march<VEC, WALLS, MODE, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMarchBytes);
+        if (e != cudaSuccess) return e;
+        configured.fetch_or(bit);
+    }
+    return launch_pdl(k_march<VEC, WALLS, MODE, PRE>, chain_grid(P.nx, P.ny, rows), dim3(kThreads), kMarchBytes, s,
+                      static_cast<const char*>(src), static_cast<char*>(dst), P, rows, fo, flag, partials);
+}
+
+template <Pass MODE, bool PRE = false>
+cudaError_t launch_march(const void* src, void* dst, const StepParams& P, int rows, FieldOut fo, unsigned* flag,
+                         double* partials, cudaStream_t s) {
+    const bool vec = (P.nx % 4) == 0;
+    const bool walls = P.wall_y != 0;
+    if (vec && walls) return launch_march_one<true, true, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
+    if (vec) return launch_march_one<true, false, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
+    if (walls) return launch_march_one<false, true, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
+    return launch_march_one<false, false, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
+}
+
 template <Pass MODE>
 cudaError_t launch_chain(const void* src, void* dst, const StepParams& P, int rows, FieldOut fo, unsigned* flag,
                          double* partials, cudaStream_t s) {
     switch (P.precision) {
         case kPrecF16: return launch_layout<LayoutF16, MODE>(src, dst, P, rows, fo, flag, partials, s);
         case kPrecB16: return launch_layout<LayoutB16, MODE>(src, dst, P, rows, fo, flag, partials, s);
-        default: return launch_layout<LayoutF32, MODE>(src, dst, P, rows, fo, flag, partials, s);
+        default: return launch_march<MODE>(src, dst, P, rows, fo, flag, partials, s);
     }
 }
 
@@ -1099,21 +1502,33 @@ dim3 chain_grid(int nx, int ny, int rows) {
 }
 
 int chain_rows(int nx, int ny, int sms, int precision) {
-    // Rows per CTA: each CTA spends (rows + 8) row-iterations (8 fill the
-    // pipeline), and the CTAs run in waves of (SMs x resident CTAs); pick
-    // the segment length that minimises waves x (rows + 8).  Short segments
-    // (1, 2, 4 rows) win on lattices too small to fill one wave.
+    // Rows per CTA.  A CTA spends rows + 7 row iterations (7 fill the
+    // pipeline); an iteration takes longer the more CTAs share its SM (FP32,
+    // 1024 columns and up: 0.75 us alone on an SM, 1.45 us with four, hence
+    // 0.55 + 0.23 n).  Within one wave the fullest SM sets the time, by a
+    // quarter more where the state is beyond L2 (2048^2: 122 us with 64 rows in
+    // one wave, 129 with 32; 4096^2: 505 us with 241 rows, 439 with 64).  Past one
+    // wave the hardware hands out CTAs as others finish, which evens out the
+    // SMs' different speeds (two dies), and half a CTA's time is lost at the
+    // end.  Measured at 8192^2: 36.3, 38.0, 40.4, 40.6, 40.9, 40.5 and 39.5
+    // GLUPS with 512, 256, 192, 128, 96, 64 and 48 rows; at 4096^2 26.8, 32.8,
+    // 36.1, 37.8, 38.2, 38.2 and 37.3 with 512, 256, 128, 96, 64, 48 and 32.
+    // The 16-bit storage keeps whole waves of two CTAs per SM and 8 fill rows.
     const int strips = (nx + kTileX - 1) / kTileX;
-    const int per_sm = precision == kPrecF32 ? pass_ctas_per_sm<LayoutF32>(Pass::Step)
-                                             : pass_ctas_per_sm<LayoutF16>(Pass::Step);
-    const long slots = static_cast<long>(per_sm) * (sms > 0 ? sms : 1);
+    const int n_sms = sms > 0 ? sms : 1;
+    const int per_sm = precision == kPrecF32 ? kMarchCtas : pass_ctas_per_sm<LayoutF16>(Pass::Step);
+    const double slots = static_cast<double>(per_sm) * n_sms;
+    const bool beyond_l2 = 144.0 * nx * ny > 126e6;
     int best = 8;
-    long best_cost = -1;
-    for (int rows = 1; rows <= 512; rows = rows < 8 ? 2 * rows : rows + 8) {
-        const long segs = (ny + rows - 1) / rows;
-        const long waves = (strips * segs + slots - 1) / slots;
-        const long cost = waves * (rows + 8);
-        if (best_cost < 0 || cost < best_cost) {
+    double best_cost = -1.0;
+    for (int rows = 1; rows <= 512; rows += rows < 32 ? 1 : 8) {
+        const long ctas = static_cast<long>(strips) * ((ny + rows - 1) / rows);
+        const double waves = ctas / slots;
+        double cost;
+        if (precision != kPrecF32) cost = std::ceil(waves) * (rows + 8);
+        else if (waves <= 1.0) cost = (rows + 7) * (0.55 + 0.23 * ((ctas + n_sms - 1) / n_sms)) * (beyond_l2 ? 1.25 : 1.0);
+        else cost = (rows + 7) * (0.55 + 0.23 * kMarchCtas) * (waves + 0.5);
+        if (best_cost < 0.0 || cost < best_cost) {
             best_cost = cost;
             best = rows;
         }
@@ -1130,7 +1545,7 @@ cudaError_t launch_step_fields(const float* src, float* dst, const StepParams& P
                                float* fwd, cudaStream_t s) {
     FieldOut fo{};
     fo.fwd = fwd;
-    return launch_layout<LayoutF32, Pass::StepFields>(src, dst, P, rows, fo, flag, nullptr, s);
+    return launch_march<Pass::StepFields>(src, dst, P, rows, fo, flag, nullptr, s);
 }
 
 cudaError_t launch_fields(const void* src, const StepParams& P, int rows, FieldOut out, cudaStream_t s) {
@@ -1143,7 +1558,7 @@ cudaError_t launch_diag_partials(const void* src, const StepParams& P, int rows,
 
 cudaError_t launch_diag_partials_pre(const float* pre, const StepParams& P, int rows, double* partials,
                                      cudaStream_t s) {
-    return launch_layout<LayoutF32, Pass::Diag, true>(pre, nullptr, P, rows, FieldOut{}, nullptr, partials, s);
+    return launch_march<Pass::Diag, true>(pre, nullptr, P, rows, FieldOut{}, nullptr, partials, s);
 }
 
 cudaError_t launch_diag_reduce(const double* partials, int nblocks, double* out, cudaStream_t s) {
