@@ -40,6 +40,7 @@
 #include <atomic>
 #include <cmath>
 #include <type_traits>
+#include <utility>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -1326,6 +1327,161 @@ __global__ void __launch_bounds__(kThreads, kMarchCtas)
     if (MODE == Pass::Diag) reduce_diag(acc, smem, partials);
 }
 
+// ---------------------------------------------------------------------------
+// Small lattices, FP32 storage: one node per thread, no marching.
+//
+// A lattice that does not fill the GPU is bound by latency: the march takes
+// rows + 7 iterations of about 0.75 us, however few its rows.  Here a CTA
+// takes a window of 32 x H nodes (26 x (H - 6) of them its own), each thread
+// gathers its node straight from L2 into registers and runs all four stages
+// of it, with three barriers and no copies in between, so that a step is one
+// load latency, four short stages and the launch.  The window's halo costs
+// 2x (H = 16) to 5x (H = 8) the arithmetic and L2 reads, which idle SMs have
+// to spare.  The arithmetic is the march's, expression by expression: both
+// give the same bits.
+// Measured per step (march -> this kernel; start of the change's tree in
+// brackets): 64^2 6.5 -> 2.05 us [5.2], 128^2 7.7 -> 2.75 [6.9], 256^2 10.3 ->
+// 4.2 [10.1], 1024 x 128 10.9 -> 7.2 [10.3], 512^2 21 -> 12.4 [22.9].
+// ---------------------------------------------------------------------------
+constexpr int kSmallX = 32;                  // window columns: one warp per window row
+constexpr int kSmallTileX = kSmallX - 6;     // output columns
+constexpr int small_tile_y(int H) { return H - 6; }
+
+template <int H, bool WALLS, Pass MODE>
+__global__ void __launch_bounds__(kSmallX * H, 1024 / (kSmallX * H))
+    k_small(const float* __restrict__ src, float* __restrict__ dst, const StepParams P, FieldOut fo,
+            unsigned* __restrict__ flag) {
+    pdl_begin();
+    constexpr int kN = kSmallX * H;
+    __shared__ float sm[7 * kN + 2 * kSmallX];
+    const int tx = threadIdx.x % kSmallX, ty = threadIdx.x / kSmallX;
+    const int nx = P.nx, ny = P.ny;
+    const size_t nodes = static_cast<size_t>(nx) * ny;
+    // this thread's node (its periodic image in the lattice)
+    const int xw = static_cast<int>(blockIdx.x) * kSmallTileX - 3 + tx;
+    const int yw = static_cast<int>(blockIdx.y) * small_tile_y(H) - 3 + ty;
+    const int x = wrap(xw, nx), y = WALLS ? yw : wrap(yw, ny);
+    const bool in = !WALLS || (y >= 0 && y < ny);
+    const bool low = WALLS && y == 0, high = WALLS && y == ny - 1;
+    float* w = sm + kSmallX + threadIdx.x;  // this node in a field of the window
+    constexpr int kChiR = 0, kChiB = 1, kPhi = 2, kNx = 3, kNy = 4, kUx = 5, kUy = 6;
+    // rows above and below in the window; beyond a wall the node's own row, odd fields negated
+    const int up = high ? 0 : kSmallX, dn = low ? 0 : -kSmallX;
+    auto dx = [&](const float* a, float pu, float pd) {
+        return ddx(a[1], a[-1], WALLS ? pu * a[up + 1] : a[up + 1], WALLS ? pu * a[up - 1] : a[up - 1],
+                   WALLS ? pd * a[dn + 1] : a[dn + 1], WALLS ? pd * a[dn - 1] : a[dn - 1]);
+    };
+    auto dy = [&](const float* a, float pu, float pd) {
+        return ddy(WALLS ? pu * a[up] : a[up], WALLS ? pd * a[dn] : a[dn], WALLS ? pu * a[up + 1] : a[up + 1],
+                   WALLS ? pu * a[up - 1] : a[up - 1], WALLS ? pd * a[dn + 1] : a[dn + 1],
+                   WALLS ? pd * a[dn - 1] : a[dn - 1]);
+    };
+    const float ou = high ? -1.0f : 1.0f, od = low ? -1.0f : 1.0f;  // parity of odd fields
+
+    // ---- A
+    float f[9], rr = 1.0f, rb = 1.0f, jx = 0.0f, jy = 0.0f, chr = 0.0f, chb = 0.0f;
+    if (in) {
+        const unsigned xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+        const unsigned ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
+        const unsigned o = static_cast<unsigned>(y) * nx + x;
+        float fr[9], fb[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            unsigned at = (lcy(i) > 0 ? ym : (lcy(i) < 0 ? yp : static_cast<unsigned>(y))) * nx +
+                          (lcx(i) > 0 ? xm : (lcx(i) < 0 ? xp : static_cast<unsigned>(x)));
+            int li = i;
+            if (WALLS && ((lcy(i) > 0 && low) || (lcy(i) < 0 && high))) {
+                li = lopp(i);
+                at = o;
+            }
+            fr[i] = __ldcg(src + nodes * li + at);
+            fb[i] = __ldcg(src + nodes * (9 + li) + at);
+        }
+        const float2 rrb = sum9x2(fr, fb);
+        rr = rrb.x;
+        rb = rrb.y;
+        jx = ((fr[1] + fb[1]) + (fr[7] + fb[7])) + (fr[8] + fb[8]) -
+             (((fr[3] + fb[3]) + (fr[5] + fb[5])) + (fr[4] + fb[4]));
+        jy = ((fr[1] + fb[1]) + (fr[3] + fb[3])) + (fr[2] + fb[2]) -
+             (((fr[5] + fb[5]) + (fr[7] + fb[7])) + (fr[6] + fb[6]));
+        const float a = rr * P.inv_rho0_r;
+        const float b = rb * P.inv_rho0_b;
+        const float inv_ab = rcp(__fadd_rn(a, b));
+        chr = a * inv_ab;
+        chb = b * inv_ab;
+        w[kChiR * kN] = chr;
+        w[kChiB * kN] = chb;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = fr[i] + fb[i];
+    }
+    const float phip = fmaf(P.phip_r, rr, P.phip_b * rb);
+    w[kPhi * kN] = phip;
+    __syncthreads();
+    // ---- B
+    float gx = 0.0f, gy = 0.0f, nhx = 0.0f, nhy = 0.0f;
+    const bool in_b = in && tx >= 1 && tx < kSmallX - 1 && ty >= 1 && ty < H - 1;
+    if (in_b) {
+        const bool use_b = chr > 0.5f;
+        const float* ch = w + (use_b ? kChiB * kN : 0);
+        const float two = use_b ? -2.0f : 2.0f;
+        gx = two * dx(ch, 1.0f, 1.0f);
+        gy = two * dy(ch, 1.0f, 1.0f);
+        const float mag2 = fmaf(gx, gx, gy * gy);
+        const float inv = (mag2 >= kNormalTau * kNormalTau) ? rsqrtf(mag2) : 0.0f;
+        nhx = -gx * inv;
+        nhy = -gy * inv;
+        w[kNx * kN] = nhx;
+        w[kNy * kN] = nhy;
+    }
+    __syncthreads();
+    // ---- C
+    float K = 0.0f, Gx = 0.0f, Gy = 0.0f, ux = 0.0f, uy = 0.0f;
+    const bool in_c = in && tx >= 2 && tx < kSmallX - 2 && ty >= 2 && ty < H - 2;
+    if (in_c) {
+        K = P.curvature_mode == 0 ? dx(w + kNx * kN, 1.0f, 1.0f) + dy(w + kNy * kN, ou, od) : P.fixed_K;
+        const float rho = rr + rb;
+        const float hk = P.half_sigma * K;
+        Gx = fmaf(hk, gx, fmaf(rho, P.gacc_x, P.gvol_x));
+        Gy = fmaf(hk, gy, fmaf(rho, P.gacc_y, P.gvol_y));
+        const float inv_rho = rcp(rho);
+        ux = fmaf(0.5f, Gx, jx) * inv_rho;
+        uy = fmaf(0.5f, Gy, jy) * inv_rho;
+        w[kUx * kN] = ux;
+        w[kUy * kN] = uy;
+    }
+    __syncthreads();
+    // ---- D
+    if (!(in && tx >= 3 && tx < kSmallX - 3 && ty >= 3 && ty < H - 3 && xw < nx && yw < ny)) return;
+    const float rho = rr + rb;
+    if (!isfinite(rho)) atomicOr(flag, 1u);
+    const float dPx = dx(w + kPhi * kN, 1.0f, 1.0f), dPy = dy(w + kPhi * kN, 1.0f, 1.0f);
+    const float divu = dx(w + kUx * kN, ou, od) + dy(w + kUy * kN, ou, od);
+    const float inv_rho = rcp(rho);
+    const float nu = node_viscosity(rr, rb, inv_rho, P);
+    float fp[9];
+    collide_increment(f, rr, rb, rho, nu, ux, uy, Gx, Gy, dPx, dPy, divu, P, fp);
+    const float ex = -nhx, ey = -nhy;
+    const float phim = fmaf(P.kphi_r, rr, P.kphi_b * rb) * inv_rho;
+    const float sg = P.beta * (rr * rb) * inv_rho * phim;
+    const size_t row = static_cast<size_t>(y) * nx;
+    store_recoloured_f32(dst + row, x, nodes, fp, rr, rb, inv_rho, sg * ex, sg * ey);
+    if (MODE == Pass::StepFields) {
+        float* o = fo.fwd + row + x;
+        o[kFwdRR * nodes] = rr;
+        o[kFwdRB * nodes] = rb;
+        o[kFwdCHR * nodes] = chr;
+        o[kFwdCHB * nodes] = chb;
+        o[kFwdPHIP * nodes] = phip;
+        o[kFwdGX * nodes] = gx;
+        o[kFwdGY * nodes] = gy;
+        o[kFwdK * nodes] = K;
+        o[kFwdGFX * nodes] = Gx;
+        o[kFwdGFY * nodes] = Gy;
+        o[kFwdUX * nodes] = ux;
+        o[kFwdUY * nodes] = uy;
+    }
+}
+
 // Batched ensemble: a persistent kernel over a work list of tiles of many
 // independent lattices.  Each CTA takes the next item (member, strip, row
 // segment) from a global counter until the list is exhausted; every item is
@@ -1470,9 +1626,59 @@ cudaError_t launch_march_one(const void* src, void* dst, const StepParams& P, in
                       static_cast<const char*>(src), static_cast<char*>(dst), P, rows, fo, flag, partials);
 }
 
+inline long small_tiles(const StepParams& P, int H) {
+    return static_cast<long>((P.nx + kSmallTileX - 1) / kSmallTileX) *
+           ((P.ny + small_tile_y(H) - 1) / small_tile_y(H));
+}
+
+// Whether a step runs as k_small.  Per step at 16 window rows: 18.3, 22.6, 29.7
+// and 40.4 us at 640^2, 720^2, 800^2 and 900^2, whatever the width; the march
+// 21.2, 24.3, 29.7 and 28.0 us with 16-byte copies and 23.1, 38, 38 and 33.6
+// us with 4-byte ones (nx not a multiple of 4).
+inline bool use_small(const StepParams& P) {
+    const long nodes = static_cast<long>(P.nx) * P.ny;
+    return nodes <= ((P.nx % 4) == 0 ? 600000 : 700000);
+}
+
+// Window rows of k_small: a step takes about 1.7 us plus c ceil(tiles / SMs),
+// c growing with the threads of a CTA (fits to 64^2 .. 512^2).
+inline int small_rows(const StepParams& P) {
+    const long sms = 152;
+    int best = 8;
+    double best_cost = 1e30;
+    for (const auto& h : {std::pair<int, double>{8, 0.45}, {10, 0.57}, {16, 1.2}}) {
+        const double cost = h.second * ((small_tiles(P, h.first) + sms - 1) / sms);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = h.first;
+        }
+    }
+    return best;
+}
+
+template <int H, Pass MODE>
+cudaError_t launch_small(const void* src, void* dst, const StepParams& P, FieldOut fo, unsigned* flag,
+                         cudaStream_t s) {
+    const dim3 g(static_cast<unsigned>((P.nx + kSmallTileX - 1) / kSmallTileX),
+                 static_cast<unsigned>((P.ny + small_tile_y(H) - 1) / small_tile_y(H)));
+    const float* a = static_cast<const float*>(src);
+    float* b = static_cast<float*>(dst);
+    if (P.wall_y) return launch_pdl(k_small<H, true, MODE>, g, dim3(kSmallX * H), 0, s, a, b, P, fo, flag);
+    return launch_pdl(k_small<H, false, MODE>, g, dim3(kSmallX * H), 0, s, a, b, P, fo, flag);
+}
+
 template <Pass MODE, bool PRE = false>
 cudaError_t launch_march(const void* src, void* dst, const StepParams& P, int rows, FieldOut fo, unsigned* flag,
                          double* partials, cudaStream_t s) {
+    if constexpr (MODE == Pass::Step || MODE == Pass::StepFields) {
+        if (use_small(P)) {
+            switch (small_rows(P)) {
+                case 8: return launch_small<8, MODE>(src, dst, P, fo, flag, s);
+                case 10: return launch_small<10, MODE>(src, dst, P, fo, flag, s);
+                default: return launch_small<16, MODE>(src, dst, P, fo, flag, s);
+            }
+        }
+    }
     const bool vec = (P.nx % 4) == 0;
     const bool walls = P.wall_y != 0;
     if (vec && walls) return launch_march_one<true, true, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
