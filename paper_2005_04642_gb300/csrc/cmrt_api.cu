@@ -111,6 +111,7 @@ struct Batch {
     cudaStream_t capture = nullptr;      // private stream on which graphs are recorded
     int precision = 0;
     bool vec = true;                     // every member has nx % 4 == 0
+    bool walls = false;                  // some member has walls
     std::vector<cmrt_params> p;
     std::vector<StepParams> sp;
     std::vector<size_t> off;
@@ -128,6 +129,9 @@ struct Batch {
     size_t items_cap = 0;
     int nitems = 0;
     int grid = 0;                        // persistent CTAs
+    int window = cmrt::kWin;             // columns of a strip's window
+    int tile() const { return window - 2 * cmrt::kHalo; }
+    cmrt::BatchForm form() const { return {precision, vec, walls, window}; }
     int diag_every = 0;                  // smallest positive diag_every of the members
     std::map<std::string, int> rows;     // size class -> rows per work item
     int graph_steps = 32;                // steps per recorded graph (even), 0 = none
@@ -1080,6 +1084,21 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 // Rows per work item before tuning: whole lattices up to 64 rows, else 64.
 int default_rows(const cmrt_params& p) { return std::min(64, std::max(1, p.ny)); }
 
+// Window width of a batch: strips of 88 or of 120 own columns, whichever
+// computes fewer window columns over all members.  512 and 256 columns take 6
+// and 3 windows of 96 (576 and 288 columns) against 5 and 3 of 128 (640 and
+// 384), 128 and 64 columns two and one of either.
+int batch_window(const std::vector<cmrt_params>& ps) {
+    double cols[2] = {0.0, 0.0};
+    const int width[2] = {96, cmrt::kWin};
+    for (const cmrt_params& p : ps)
+        for (int k = 0; k < 2; ++k) {
+            const int tile = width[k] - 2 * cmrt::kHalo;
+            cols[k] += static_cast<double>((p.nx + tile - 1) / tile) * width[k] * p.ny;
+        }
+    return cols[0] < cols[1] ? width[0] : width[1];
+}
+
 Batch* blive(cmrt_batch* h) {
     if (!h) {
         bfail(nullptr, CMRT_ESTATE, "NULL batch");
@@ -1125,7 +1144,7 @@ void free_batch(Batch* b) {
 }
 
 // Work list for the current rows per class: every member cut into strips of
-// kTileX columns and segments of its class's rows, longest segments first,
+// the batch's tile width and segments of its class's rows, longest segments first,
 // and within equal lengths member by member, segment by segment, so that
 // neighbouring strips (which share halo columns) run close together in time.
 cmrt_status build_items(Batch* b) {
@@ -1133,10 +1152,10 @@ cmrt_status build_items(Batch* b) {
     for (int m = 0; m < b->n; ++m) {
         const cmrt_params& p = b->p[m];
         const int r = b->rows[class_key(p)];
-        const int strips = (p.nx + cmrt::kTileX - 1) / cmrt::kTileX;
+        const int strips = (p.nx + b->tile() - 1) / b->tile();
         for (int y0 = 0; y0 < p.ny; y0 += r)
             for (int s = 0; s < strips; ++s)
-                items.push_back(cmrt::BatchItem{m, s * cmrt::kTileX, y0, std::min(r, p.ny - y0)});
+                items.push_back(cmrt::BatchItem{m, s * b->tile(), y0, std::min(r, p.ny - y0)});
     }
     std::stable_sort(items.begin(), items.end(),
                      [](const cmrt::BatchItem& a, const cmrt::BatchItem& c) { return a.rows > c.rows; });
@@ -1170,7 +1189,7 @@ cudaError_t batch_launch(Batch* b, int src_parity, cudaStream_t s) {
     cmrt::BatchArgs A{b->d_items, b->nitems, b->d_params, b->d_off,
                       static_cast<const char*>(b->buf[src_parity]), static_cast<char*>(b->buf[src_parity ^ 1]),
                       b->d_flags, b->d_counters};
-    return cmrt::launch_batch(A, b->precision, b->vec, b->grid, s);
+    return cmrt::launch_batch(A, b->form(), b->grid, s);
 }
 
 // Records graph_steps batched steps starting from buffer parity `parity`.
@@ -1324,6 +1343,7 @@ cmrt_status cmrt_batch_init(int32_t n, const cmrt_params* params, const float* c
     for (int m = 0; m < n; ++m) {
         b->sp.push_back(derive(params[m]));
         b->vec = b->vec && (params[m].nx % 4) == 0;
+        b->walls = b->walls || params[m].wall_y != 0;
         b->off.push_back(b->arena_bytes);
         const size_t bytes = static_cast<size_t>(params[m].nx) * params[m].ny * node;
         b->arena_bytes += (bytes + 255) / 256 * 256;  // 256-byte aligned members
@@ -1361,8 +1381,9 @@ cmrt_status cmrt_batch_init(int32_t n, const cmrt_params* params, const float* c
         !ck(cudaMemsetAsync(b->d_flags, 0, n * sizeof(unsigned), b->stream), "cudaMemsetAsync") ||
         !ck(cudaMemsetAsync(b->d_counters, 0, 2 * sizeof(unsigned), b->stream), "cudaMemsetAsync"))
         return bail(CMRT_ECUDA);
+    b->window = batch_window(b->p);
     int per_sm = 0, sms = 0;
-    if (!ck(cmrt::prepare_batch(b->precision, b->vec, &per_sm), "setting up the batched kernel") ||
+    if (!ck(cmrt::prepare_batch(b->form(), &per_sm), "setting up the batched kernel") ||
         !ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device), "cudaDeviceGetAttribute"))
         return bail(CMRT_ECUDA);
     if (per_sm < 1) {

@@ -96,7 +96,6 @@ constexpr int kThreads = 128;
 constexpr int kWin = 128;
 constexpr int kHalo = 4;
 constexpr int kTileX = kWin - 2 * kHalo;  // 120
-constexpr int kRing = 9;                  // rows of post-collision populations kept in shared memory
 
 // Step: one time step; StepFields: the same step, also writing the forward
 // fields of its input state (FP32 storage, for the adjoint's segment replay).
@@ -121,6 +120,11 @@ cudaError_t launch_step(const void* src, void* dst, const StepParams& P, int row
 // the values the adjoint's own forward recomputation gives.
 cudaError_t launch_step_fields(const float* src, float* dst, const StepParams& P, int rows, unsigned* flag,
                                float* fwd, cudaStream_t s);
+// The passes of a lattice with 16-bit storage (cmrt_step16.cu), which the three
+// calls around them hand over to.
+cudaError_t launch_step16(const void* src, void* dst, const StepParams& P, int rows, unsigned* flag, cudaStream_t s);
+cudaError_t launch_fields16(const void* src, const StepParams& P, int rows, FieldOut out, cudaStream_t s);
+cudaError_t launch_diag_partials16(const void* src, const StepParams& P, int rows, double* partials, cudaStream_t s);
 // Fields of the state whose post-collision populations are in src.
 cudaError_t launch_fields(const void* src, const StepParams& P, int rows, FieldOut out, cudaStream_t s);
 // Per-CTA FP64 partial diagnostics into partials[grid][kDiagSlots].
@@ -131,7 +135,7 @@ cudaError_t launch_diag_partials_pre(const float* pre, const StepParams& P, int 
 // Reduces nblocks partial rows into out[kDiagSlots] (one CTA).
 cudaError_t launch_diag_reduce(const double* partials, int nblocks, double* out, cudaStream_t s);
 
-// Batched ensembles: one work item is the strip [x0, x0 + kTileX) of rows
+// Batched ensembles: one work item is the strip of columns from x0 of rows
 // [y0, y0 + rows) of lattice `member`.
 struct BatchItem {
     int member, x0, y0, rows;
@@ -149,11 +153,19 @@ struct BatchArgs {
     unsigned* counters;         // [2] next item, CTAs finished; zero between launches
 };
 
-// Sets up the batched kernel for a storage precision on the current device
-// and reports how many of its CTAs fit on one SM.
-cudaError_t prepare_batch(int precision, bool vec, int* ctas_per_sm);
+// What the batched kernel is compiled for: storage, 16-byte copies (every nx a
+// multiple of 4), whether any member has walls, and the columns of a strip's
+// window (96 or kWin, of which all but 2 kHalo are the strip's own).
+struct BatchForm {
+    int precision;
+    bool vec, walls;
+    int window;
+};
+// Sets up the batched kernel on the current device and reports how many of its
+// CTAs fit on one SM.
+cudaError_t prepare_batch(const BatchForm& b, int* ctas_per_sm);
 // One step of every member of a batch: `grid` persistent CTAs drain the work list.
-cudaError_t launch_batch(const BatchArgs& A, int precision, bool vec, int grid, cudaStream_t s);
+cudaError_t launch_batch(const BatchArgs& A, const BatchForm& b, int grid, cudaStream_t s);
 
 // Plane passes (cmrt_planes.cu), FP32 storage: one thread per node, the
 // intermediate fields in scratch planes float[kAdjPlanes][ny][nx].
