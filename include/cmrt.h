@@ -123,9 +123,10 @@ typedef struct {
                                 forward steps can write the forward fields the reverse steps read
                                 (one set of 14 planes per recomputed or kept state, allocated where
                                 memory allows); otherwise, and in cmrt_step_vjp, the fused kernels
-                                where the lattice fills 16-row segments in two waves of the GPU and
-                                eight per-node plane passes on smaller lattices; 1 = always the
-                                fused kernels; 2 = always the plane passes.  Both compute the same
+                                where the lattice fills 16-row segments in two waves of the GPU or
+                                is small enough for their one-node-per-thread form (400 000 nodes,
+                                900 000 in cmrt_step_vjp) and eight per-node plane passes in
+                                between; 1 = always the fused kernels; 2 = always the plane passes.  Both compute the same
                                 values (rounding order aside)                                     */
 } cmrt_params;
 

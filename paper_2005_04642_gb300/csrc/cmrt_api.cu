@@ -415,13 +415,11 @@ cmrt_status check_flag(Ctx* c) {
     return CMRT_OK;
 }
 
-// One step src -> dst: the fused kernel, or the plane passes for the order-6
-// stencil.  Returns the number of kernels launched, or -1 on a launch error.
+// One step src -> dst: the fused kernel of either stencil.  Returns the number of kernels launched, or -1 on a launch error.
 int step_once(Ctx* c, const void* src, void* dst, cudaError_t* err) {
     if (c->p.stencil_order == 6) {
-        *err = cmrt::launch_step_planes(static_cast<const float*>(src), static_cast<float*>(dst), c->sp,
-                                        c->adj_scratch, c->d_flag, c->stream);
-        return *err == cudaSuccess ? 4 : -1;
+        *err = cmrt::launch_step6(static_cast<const float*>(src), static_cast<float*>(dst), c->sp, c->d_flag, c->stream);
+        return *err == cudaSuccess ? 1 : -1;
     }
     *err = cmrt::launch_step(src, dst, c->sp, c->rows, c->d_flag, c->stream);
     return *err == cudaSuccess ? 1 : -1;
@@ -473,12 +471,11 @@ cmrt_status build_step_graph(Ctx* c, int parity) {
 // n plain steps on the context's stream: whole graphs of graph_steps steps
 // (an even count, so the buffer parity is unchanged), then single launches.
 cmrt_status advance(Ctx* c, int64_t n) {
-    const int per_step = c->p.stencil_order == 6 ? 4 : 1;
     while (c->graph_steps > 0 && n >= c->graph_steps) {
         if (!c->step_exec[c->cur] && build_step_graph(c, c->cur) != CMRT_OK) return CMRT_ECUDA;
         CK(c, cudaGraphLaunch(c->step_exec[c->cur], c->stream));
         c->t += c->graph_steps;
-        c->launches += static_cast<int64_t>(c->graph_steps) * per_step;
+        c->launches += c->graph_steps;
         n -= c->graph_steps;
     }
     for (; n > 0; --n) {
@@ -615,19 +612,7 @@ cmrt_status cmrt_init(const cmrt_params* p, const float* rho_n0, const float* u0
     c->rows = cmrt::chain_rows(p->nx, p->ny, sms, p->precision);
     const dim3 g = cmrt::chain_grid(p->nx, p->ny, c->rows);
     c->n_partials = static_cast<int>(g.x * g.y);
-    if (p->stencil_order == 6) {
-        // the order-6 passes keep their fields in the scratch planes and write
-        // one partial row per 128-column block of a lattice row
-        c->n_partials = std::max(c->n_partials, cmrt::adj_blocks(p->nx, p->ny));
-        const size_t bytes = cmrt::kAdjPlanes * cells(*c) * sizeof(float);
-        if (cudaMalloc(&c->adj_scratch, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            c->adj_scratch = nullptr;
-            fail(c, CMRT_ENOMEM, "cudaMalloc of %zu scratch bytes for the order-6 step failed", bytes);
-            return bail(CMRT_ENOMEM);
-        }
-        c->adj_bytes += bytes;
-    }
+    if (p->stencil_order == 6) c->n_partials = cmrt::diag_blocks6(p->nx, p->ny);
     if (cudaMalloc(&c->d_flag, sizeof(unsigned)) != cudaSuccess ||
         cudaMalloc(&c->d_partials, sizeof(double) * cmrt::kDiagSlots * c->n_partials) != cudaSuccess ||
         cudaMalloc(&c->d_diag, sizeof(double) * cmrt::kDiagSlots) != cudaSuccess) {
@@ -716,13 +701,11 @@ cmrt_status cmrt_fields(cmrt_ctx* h, float* rho_r, float* rho_b, float* ux, floa
     }
     const cmrt::FieldOut fo{dev[0], dev[1], dev[2], dev[3], dev[4]};
     if (c->p.stencil_order == 6) {
-        CK(c, cmrt::launch_fields_planes(static_cast<const float*>(c->buf[c->cur]), c->sp, c->adj_scratch, fo,
-                                         c->stream));
-        c->launches += 4;
+        CK(c, cmrt::launch_fields6(static_cast<const float*>(c->buf[c->cur]), c->sp, fo, c->stream));
     } else {
         CK(c, cmrt::launch_fields(c->buf[c->cur], c->sp, c->rows, fo, c->stream));
-        c->launches++;
     }
+    c->launches++;
     if (any_host) {
         for (int k = 0; k < 5; ++k)
             if (copy[k]) CK(c, cudaMemcpyAsync(outs[k], dev[k], n * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
@@ -738,15 +721,12 @@ cmrt_status cmrt_diagnostics(cmrt_ctx* h, double out[6]) {
     if (!out) return fail(c, CMRT_EINVAL, "out is NULL");
     if (set_device(c) != CMRT_OK) return CMRT_ECUDA;
     if (c->p.stencil_order == 6) {
-        CK(c, cmrt::launch_diag_planes(static_cast<const float*>(c->buf[c->cur]), c->sp, c->adj_scratch,
-                                       c->d_partials, c->stream));
-        CK(c, cmrt::launch_diag_reduce(c->d_partials, cmrt::adj_blocks(c->p.nx, c->p.ny), c->d_diag, c->stream));
-        c->launches += 5;
+        CK(c, cmrt::launch_diag6(static_cast<const float*>(c->buf[c->cur]), c->sp, c->d_partials, c->stream));
     } else {
         CK(c, cmrt::launch_diag_partials(c->buf[c->cur], c->sp, c->rows, c->d_partials, c->stream));
-        CK(c, cmrt::launch_diag_reduce(c->d_partials, c->n_partials, c->d_diag, c->stream));
-        c->launches += 2;
     }
+    CK(c, cmrt::launch_diag_reduce(c->d_partials, c->n_partials, c->d_diag, c->stream));
+    c->launches += 2;
     double h6[cmrt::kDiagSlots];
     CK(c, cudaMemcpyAsync(h6, c->d_diag, sizeof h6, cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
@@ -953,7 +933,7 @@ extern "C" cmrt_status cmrt_diagnostics_noalloc(const cmrt_params* p, const floa
     if (st != CMRT_OK) return st;
     if (!pops || !out) return fail(nullptr, CMRT_EINVAL, "pops and out must not be NULL");
     if (p->stencil_order != 2)
-        return fail(nullptr, CMRT_EINVAL, "stencil_order 6 needs a context (its passes keep fields in scratch planes)");
+        return fail(nullptr, CMRT_EINVAL, "stencil_order 6 needs a context");
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
         cudaGetLastError();
@@ -1734,9 +1714,9 @@ cmrt_status ensure_adj(Ctx* c, size_t ckpt, size_t seg, size_t fields) {
     return CMRT_OK;
 }
 
-// Reduces the partial sums into out[kAdjSlots] on the host (synchronises).
-cmrt_status adj_collect(Ctx* c, double* out) {
-    CK(c, cmrt::launch_adjoint_reduce(c->adj_partials, cmrt::adj_blocks(c->p.nx, c->p.ny), c->adj_out, c->stream));
+// Reduces `blocks` rows of the partial sums into out[kAdjSlots] on the host (synchronises).
+cmrt_status adj_collect(Ctx* c, int blocks, double* out) {
+    CK(c, cmrt::launch_adjoint_reduce(c->adj_partials, blocks, c->adj_out, c->stream));
     c->launches++;
     CK(c, cudaMemcpyAsync(out, c->adj_out, cmrt::kAdjSlots * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
@@ -1762,22 +1742,34 @@ extern "C" cmrt_status cmrt_step_vjp(cmrt_ctx* h, const float* lam_next, float* 
     cmrt_status st = ensure_adj(c, 0, 0, 0);
     if (st != CMRT_OK) return st;
     const size_t n18 = cells(*c) * 18;
-    const float* src = lam_next;
-    if (!is_device_ptr(lam_next)) {
-        CK(c, cudaMemcpyAsync(c->adj_lam[1], lam_next, n18 * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-        src = c->adj_lam[1];
-    }
-    // adjoint of P_t: the transpose of the gather f(t+1) = gather(P_t), a permutation
-    CK(c, cmrt::launch_unstream_in(src, c->sp, c->adj_lam[0], c->stream));
-    if ((st = adj_zero(c)) != CMRT_OK) return st;
+    const bool small = cmrt::adj_vjp_small(c->sp);
     const bool host = !is_device_ptr(lam);
     float* dst = host ? c->adj_lam[1] : lam;
-    CK(c, cmrt::launch_adjoint_step_pre(static_cast<const float*>(c->buf[c->cur]), c->adj_lam[0], c->sp,
-                                        c->adj_scratch, c->adj_partials, dst, c->stream));
-    c->launches += 1 + cmrt::adj_launches_per_step(c->sp);
+    const float* src = lam_next;
+    // lam_next in a buffer of the library: from the host, or where lam overlaps
+    // it, since the window kernels read it at neighbours while lam is written
+    if (!is_device_ptr(lam_next) || (small && src < dst + n18 && dst < src + n18)) {
+        float* in = small ? c->adj_lam[0] : c->adj_lam[1];
+        CK(c, cudaMemcpyAsync(in, lam_next, n18 * sizeof(float), cudaMemcpyDefault, c->stream));
+        src = in;
+    }
+    const float* post = static_cast<const float*>(c->buf[c->cur]);
+    const int all = cmrt::adj_blocks(c->p.nx, c->p.ny);
+    const int blocks = small ? cmrt::adj_vjp_small_blocks(c->sp) : all;
+    if (blocks == all && (st = adj_zero(c)) != CMRT_OK) return st;
+    if (small) {
+        CK(c, cmrt::launch_vjp_small(post, src, c->sp, c->adj_scratch, c->adj_partials, dst, c->stream));
+    } else {
+        // adjoint of P_t: the transpose of the gather f(t+1) = gather(P_t), a permutation
+        CK(c, cmrt::launch_unstream_in(src, c->sp, c->adj_lam[0], c->stream));
+        CK(c, cmrt::launch_adjoint_step_pre(post, c->adj_lam[0], c->sp, c->adj_scratch, c->adj_partials, dst,
+                                            c->stream));
+        c->launches++;
+    }
+    c->launches += cmrt::adj_launches_per_step(c->sp, true);
     if (host) CK(c, cudaMemcpyAsync(lam, dst, n18 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     double out[cmrt::kAdjSlots];
-    if ((st = adj_collect(c, out)) != CMRT_OK) return st;
+    if ((st = adj_collect(c, blocks, out)) != CMRT_OK) return st;
     if (grad_params)
         for (int k = 0; k < 6; ++k) grad_params[k] += out[k];
     return CMRT_OK;
@@ -1956,7 +1948,7 @@ extern "C" cmrt_status cmrt_adjoint(cmrt_ctx* h, int64_t nsteps, int32_t ckpt_ev
         if (host) CK(c, cudaMemcpyAsync(grad_rho_n0, g, n * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     }
     double out[cmrt::kAdjSlots];
-    if ((st = adj_collect(c, out)) != CMRT_OK) return st;
+    if ((st = adj_collect(c, cmrt::adj_blocks(c->p.nx, c->p.ny), out)) != CMRT_OK) return st;
     if (J) *J = out[6];
     if (grad_params)
         for (int k = 0; k < 6; ++k) grad_params[k] = out[k];

@@ -99,7 +99,8 @@ constexpr int kTileX = kWin - 2 * kHalo;  // 120
 
 // Step: one time step; StepFields: the same step, also writing the forward
 // fields of its input state (FP32 storage, for the adjoint's segment replay).
-enum class Pass : int { Step = 0, Fields = 1, Diag = 2, StepFields = 3 };
+// FwdFields: those forward fields alone (small lattices).
+enum class Pass : int { Step = 0, Fields = 1, Diag = 2, StepFields = 3, FwdFields = 4 };
 
 // Number of FP64 partial sums each CTA of the diagnostics pass writes.
 constexpr int kDiagSlots = 6;  // mass_r, mass_b, mom_x, mom_y, max|u|^2, non-finite count
@@ -125,6 +126,9 @@ cudaError_t launch_step_fields(const float* src, float* dst, const StepParams& P
 cudaError_t launch_step16(const void* src, void* dst, const StepParams& P, int rows, unsigned* flag, cudaStream_t s);
 cudaError_t launch_fields16(const void* src, const StepParams& P, int rows, FieldOut out, cudaStream_t s);
 cudaError_t launch_diag_partials16(const void* src, const StepParams& P, int rows, double* partials, cudaStream_t s);
+// The forward fields alone (lattices the small-lattice kernel takes, FP32
+// storage), the same bits as launch_step_fields.
+cudaError_t launch_fwd_fields(const float* src, const StepParams& P, float* fwd, cudaStream_t s);
 // Fields of the state whose post-collision populations are in src.
 cudaError_t launch_fields(const void* src, const StepParams& P, int rows, FieldOut out, cudaStream_t s);
 // Per-CTA FP64 partial diagnostics into partials[grid][kDiagSlots].
@@ -167,16 +171,13 @@ cudaError_t prepare_batch(const BatchForm& b, int* ctas_per_sm);
 // One step of every member of a batch: `grid` persistent CTAs drain the work list.
 cudaError_t launch_batch(const BatchArgs& A, const BatchForm& b, int grid, cudaStream_t s);
 
-// Plane passes (cmrt_planes.cu), FP32 storage: one thread per node, the
-// intermediate fields in scratch planes float[kAdjPlanes][ny][nx].
-// The step, fields and diagnostics with the order-6 gradient (App. B); each
-// launches 4 kernels, diagnostics write partials[adj_blocks][kDiagSlots].
-cudaError_t launch_step_planes(const float* post, float* dst, const StepParams& P, float* scratch, unsigned* flag,
-                               cudaStream_t s);
-cudaError_t launch_fields_planes(const float* post, const StepParams& P, float* scratch, FieldOut out,
-                                 cudaStream_t s);
-cudaError_t launch_diag_planes(const float* post, const StepParams& P, float* scratch, double* partials,
-                               cudaStream_t s);
+// The step, fields and diagnostics with the order-6 gradient of App. B
+// (cmrt_order6.cu), FP32 storage, one launch each; the diagnostics write
+// partials[diag_blocks6][kDiagSlots].
+cudaError_t launch_step6(const float* src, float* dst, const StepParams& P, unsigned* flag, cudaStream_t s);
+cudaError_t launch_fields6(const float* src, const StepParams& P, FieldOut out, cudaStream_t s);
+int diag_blocks6(int nx, int ny);
+cudaError_t launch_diag6(const float* src, const StepParams& P, double* partials, cudaStream_t s);
 
 // Discrete adjoint (cmrt_planes.cu), FP32 storage.  scratch: float[kAdjPlanes][ny][nx];
 // partials: double[adj_blocks][kAdjSlots], accumulated by every launch (zero it
@@ -185,7 +186,9 @@ cudaError_t launch_diag_planes(const float* post, const StepParams& P, float* sc
 constexpr int kAdjPlanes = 38;
 constexpr int kAdjSlots = 8;
 int adj_blocks(int nx, int ny);
-int adj_launches_per_step(const StepParams& P);
+// kernels of one reverse step that recomputes the forward fields (vjp: of a
+// step VJP)
+int adj_launches_per_step(const StepParams& P, bool vjp = false);
 // lam_post: adjoint of P_t; post: P_{t-1}; writes the adjoint of P_{t-1} into lam_prev.
 // fwd: the forward fields of post written by launch_step_fields, or null to
 // recompute them (used only where adj_fused(P)).
@@ -197,6 +200,13 @@ bool adj_fused(const StepParams& P);
 // steps (compact stencil, plane passes not asked for); a call that uses such
 // fields runs all its reverse steps fused
 bool adj_fields_usable(const StepParams& P);
+// cmrt_step_vjp by windows (small lattices): lam_next is dJ/df(t+1) and lam
+// receives dJ/df(t), both in the public layout.  The rows of partials used:
+// written, where they are fewer than adj_blocks, else added to.
+bool adj_vjp_small(const StepParams& P);
+int adj_vjp_small_blocks(const StepParams& P);
+cudaError_t launch_vjp_small(const float* post, const float* lam_next, const StepParams& P, float* scratch,
+                             double* partials, float* lam, cudaStream_t s);
 // same, but writes dJ/df(t) (pre-collision, float[2][9][ny][nx]) into lam_pre
 cudaError_t launch_adjoint_step_pre(const float* post, const float* lam_post, const StepParams& P, float* scratch,
                                     double* partials, float* lam_pre, cudaStream_t s);

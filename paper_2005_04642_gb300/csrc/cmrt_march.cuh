@@ -990,24 +990,8 @@ __global__ void __launch_bounds__(kSmallX * H, 1024 / (kSmallX * H))
     __syncthreads();
     // ---- D
     if (!(in && tx >= kEdge && tx < kSmallX - kEdge && ty >= kEdge && ty < H - kEdge && xw < nx && yw < ny)) return;
-    const float rho = rr + rb;
-    if (!isfinite(rho)) atomicOr(flag, 1u);
-    const float dPx = dx(w + kPhi * kN, 1.0f, 1.0f), dPy = dy(w + kPhi * kN, 1.0f, 1.0f);
-    const float divu = dx(w + kUx * kN, ou, od) + dy(w + kUy * kN, ou, od);
-    const float inv_rho = rcp(rho);
-    const float nu = node_viscosity(rr, rb, inv_rho, P);
-    float fp[9];
-    collide_increment(f, rr, rb, rho, nu, ux, uy, Gx, Gy, dPx, dPy, divu, P, fp);
-    const float ex = -nhx, ey = -nhy;
-    const float phim = fmaf(P.kphi_r, rr, P.kphi_b * rb) * inv_rho;
-    const float sg = P.beta * (rr * rb) * inv_rho * phim;
     const size_t row = static_cast<size_t>(y) * nx;
-    if constexpr (L::kDecode)
-        L::Record::store(dst, nodes, row, x, fp, rr, rb, inv_rho, sg * ex, sg * ey, fmaf(0.5f * Gx, inv_rho, ux),
-                         fmaf(0.5f * Gy, inv_rho, uy), P);
-    else
-        store_recoloured_f32(reinterpret_cast<float*>(dst) + row, x, nodes, fp, rr, rb, inv_rho, sg * ex, sg * ey);
-    if (MODE == Pass::StepFields) {
+    if (MODE == Pass::StepFields || MODE == Pass::FwdFields) {
         float* o = fo.fwd + row + x;
         o[kFwdRR * nodes] = rr;
         o[kFwdRB * nodes] = rb;
@@ -1021,7 +1005,24 @@ __global__ void __launch_bounds__(kSmallX * H, 1024 / (kSmallX * H))
         o[kFwdGFY * nodes] = Gy;
         o[kFwdUX * nodes] = ux;
         o[kFwdUY * nodes] = uy;
+        if (MODE == Pass::FwdFields) return;
     }
+    const float rho = rr + rb;
+    if (!isfinite(rho)) atomicOr(flag, 1u);
+    const float dPx = dx(w + kPhi * kN, 1.0f, 1.0f), dPy = dy(w + kPhi * kN, 1.0f, 1.0f);
+    const float divu = dx(w + kUx * kN, ou, od) + dy(w + kUy * kN, ou, od);
+    const float inv_rho = rcp(rho);
+    const float nu = node_viscosity(rr, rb, inv_rho, P);
+    float fp[9];
+    collide_increment(f, rr, rb, rho, nu, ux, uy, Gx, Gy, dPx, dPy, divu, P, fp);
+    const float ex = -nhx, ey = -nhy;
+    const float phim = fmaf(P.kphi_r, rr, P.kphi_b * rb) * inv_rho;
+    const float sg = P.beta * (rr * rb) * inv_rho * phim;
+    if constexpr (L::kDecode)
+        L::Record::store(dst, nodes, row, x, fp, rr, rb, inv_rho, sg * ex, sg * ey, fmaf(0.5f * Gx, inv_rho, ux),
+                         fmaf(0.5f * Gy, inv_rho, uy), P);
+    else
+        store_recoloured_f32(reinterpret_cast<float*>(dst) + row, x, nodes, fp, rr, rb, inv_rho, sg * ex, sg * ey);
 }
 
 template <class L, bool VEC, bool WALLS, Pass MODE, bool PRE>
@@ -1057,7 +1058,8 @@ template <class L>
 bool use_small(const StepParams& P) {
     const long nodes = static_cast<long>(P.nx) * P.ny;
     const long limit = L::kDecode ? 450000 : 600000;
-    return nodes <= ((P.nx % 4) == 0 ? limit : limit + 100000);
+    const int rows = 16 - 2 * small_halo<L>();
+    return nodes <= ((P.nx % 4) == 0 ? limit : limit + 100000) && P.ny <= 65535 * rows;  // grid rows
 }
 
 // Window rows of k_small: a step takes about 1.7 us plus c ceil(tiles / SMs),
@@ -1076,7 +1078,7 @@ int small_rows(const StepParams& P) {
         if (f.rows <= 2 * small_halo<L>()) continue;  // no rows of its own
         const dim3 g = small_grid<L>(P, f.rows);
         const double cost = f.c * ((static_cast<long>(g.x) * g.y + sms - 1) / sms);
-        if (cost < best_cost) {
+        if (cost < best_cost && g.y <= 65535) {
             best_cost = cost;
             best = f.rows;
         }
@@ -1094,19 +1096,23 @@ cudaError_t launch_small(const void* src, void* dst, const StepParams& P, FieldO
     return launch_pdl(k_small<L, H, false, MODE>, g, dim3(kSmallX * H), 0, s, a, b, P, fo, flag);
 }
 
+template <class L, Pass MODE>
+cudaError_t launch_small_any(const void* src, void* dst, const StepParams& P, FieldOut fo, unsigned* flag,
+                             cudaStream_t s) {
+    switch (small_rows<L>(P)) {
+        case 8:
+            if constexpr (!L::kDecode) return launch_small<L, 8, MODE>(src, dst, P, fo, flag, s);
+            [[fallthrough]];
+        case 10: return launch_small<L, 10, MODE>(src, dst, P, fo, flag, s);
+        default: return launch_small<L, 16, MODE>(src, dst, P, fo, flag, s);
+    }
+}
+
 template <class L, Pass MODE, bool PRE = false>
 cudaError_t launch_march(const void* src, void* dst, const StepParams& P, int rows, FieldOut fo, unsigned* flag,
                          double* partials, cudaStream_t s) {
     if constexpr (MODE == Pass::Step || MODE == Pass::StepFields) {
-        if (use_small<L>(P)) {
-            switch (small_rows<L>(P)) {
-                case 8:
-                    if constexpr (!L::kDecode) return launch_small<L, 8, MODE>(src, dst, P, fo, flag, s);
-                    [[fallthrough]];
-                case 10: return launch_small<L, 10, MODE>(src, dst, P, fo, flag, s);
-                default: return launch_small<L, 16, MODE>(src, dst, P, fo, flag, s);
-            }
-        }
+        if (use_small<L>(P)) return launch_small_any<L, MODE>(src, dst, P, fo, flag, s);
     }
     const bool vec = (P.nx % 4) == 0;
     const bool walls = P.wall_y != 0;

@@ -1,0 +1,244 @@
+// The step, fields and diagnostics with App. B's order-6 colour and Phi'
+// gradients (arXiv 2005.04642), FP32 storage:
+//   d_a X = sum_N a_N sum_i w_i X(r + N c_i) c_ia,  (a_1, a_2, a_3) = (9/2, -9/10, 1/10),
+// a stencil of radius 3, with the compact one for K and div u.
+//
+// One node per thread: a CTA takes a window of 32 x H nodes, 22 x (H - 10) of
+// them its own, gathers each node's populations into registers and runs
+//   moments, chi, Phi' | grad rho^N, n-hat (halo 2) | K, G, u (halo 1) | the rest,
+// with a barrier between, the fields that a stencil reads in shared memory.
+// What bounds it: the launch and one load latency on small lattices, else
+// latency at one CTA of 1024 threads per SM (the window's halo makes the moments
+// 2x, H = 32, to 4x their work; whole warps of halo rows skip the collision).
+// Per step, as four passes over planes in memory -> here: 64^2 9.2 -> 2.7 us,
+// 256^2 11.2 -> 5.2, 512^2 21.4 -> 18.3, 1024 x 512 38.2 -> 34.2, 2048^2 302 ->
+// 279; one launch instead of four, and no 28 planes of scratch per node.
+#include <atomic>
+
+#include "cmrt_device.cuh"
+
+namespace cmrt {
+namespace {
+
+constexpr int kX = 32, kEdge = 5;
+
+__device__ __forceinline__ int wrap(int v, int n) {
+    if (v >= 0 && v < n) return v;
+    const int r = v % n;
+    return r < 0 ? r + n : r;
+}
+// App. B coefficients a_N
+__host__ __device__ constexpr float coef(int N) { return N == 1 ? 4.5f : (N == 2 ? -0.9f : 0.1f); }
+
+template <int H, bool W, Pass MODE>
+__global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
+    k_order6(const float* __restrict__ src, float* __restrict__ dst, const StepParams P, FieldOut fo,
+             unsigned* __restrict__ flag, double* __restrict__ partials) {
+    pdl_begin();
+    constexpr int kN = kX * H;
+    __shared__ float sm[7 * kN + 2 * kX];
+    const int tx = threadIdx.x % kX, ty = threadIdx.x / kX;
+    const int nx = P.nx, ny = P.ny;
+    const size_t nodes = static_cast<size_t>(nx) * ny;
+    const int xw = static_cast<int>(blockIdx.x) * (kX - 2 * kEdge) - kEdge + tx;
+    const int yw = static_cast<int>(blockIdx.y) * (H - 2 * kEdge) - kEdge + ty;
+    const int x = wrap(xw, nx), y = W ? yw : wrap(yw, ny);
+    const bool in = !W || (y >= 0 && y < ny);
+    auto inner = [&](int d) { return in && tx >= d && tx < kX - d && ty >= d && ty < H - d; };
+    const bool own = inner(kEdge) && xw < nx && yw < ny;
+    const bool low = W && y == 0, high = W && y == ny - 1;
+    float* w = sm + kX + threadIdx.x;  // this node in a field of the window
+    constexpr int kChiR = 0, kChiB = 1, kPhi = 2, kNx = 3, kNy = 4, kUx = 5, kUy = 6;
+    // window offset of the row y + dy, or of its mirror beyond a wall
+    auto row = [&](int dy) {
+        int t = y + dy;
+        if (W && t < 0) t = -1 - t;
+        if (W && t >= ny) t = 2 * ny - 1 - t;
+        return W ? (t - y) * kX : dy * kX;
+    };
+    auto grad6 = [&](const float* a, float& gx, float& gy) {
+        gx = 0.0f;
+        gy = 0.0f;
+#pragma unroll
+        for (int N = 1; N <= 3; ++N) {
+            const int rows[3] = {row(-N), 0, row(N)};
+#pragma unroll
+            for (int i = 1; i < 9; ++i) {
+                const float v = a[rows[lcy(i) + 1] + N * lcx(i)];
+                if (lcx(i)) gx = fmaf(coef(N) * lw(i) * float(lcx(i)), v, gx);
+                if (lcy(i)) gy = fmaf(coef(N) * lw(i) * float(lcy(i)), v, gy);
+            }
+        }
+    };
+    // compact derivatives: beyond a wall the node's own row times the field's parity
+    const int up = high ? 0 : kX, dn = low ? 0 : -kX;
+    auto d_x = [&](const float* a, float parity) {
+        const float pu = high ? parity : 1.0f, pd = low ? parity : 1.0f;
+        return ddx(a[1], a[-1], pu * a[up + 1], pu * a[up - 1], pd * a[dn + 1], pd * a[dn - 1]);
+    };
+    auto d_y = [&](const float* a, float parity) {
+        const float pu = high ? parity : 1.0f, pd = low ? parity : 1.0f;
+        return ddy(pu * a[up], pd * a[dn], pu * a[up + 1], pu * a[up - 1], pd * a[dn + 1], pd * a[dn - 1]);
+    };
+
+    // ---- moments, colour fractions, Phi'
+    float f[9], rr = 1.0f, rb = 1.0f, jx = 0.0f, jy = 0.0f, chr = 0.0f, chb = 0.0f;
+    if (in) {
+        const unsigned xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+        const unsigned ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
+        float fr[9], fb[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            unsigned at = (lcy(i) > 0 ? ym : (lcy(i) < 0 ? yp : static_cast<unsigned>(y))) * nx +
+                          (lcx(i) > 0 ? xm : (lcx(i) < 0 ? xp : static_cast<unsigned>(x)));
+            int li = i;
+            if (W && ((lcy(i) > 0 && low) || (lcy(i) < 0 && high))) {  // half-way bounce-back
+                li = lopp(i);
+                at = static_cast<unsigned>(y) * nx + x;
+            }
+            fr[i] = __ldcg(src + nodes * li + at);
+            fb[i] = __ldcg(src + nodes * (9 + li) + at);
+        }
+        rr = ((fr[0] + fr[1]) + (fr[2] + fr[3])) + ((fr[4] + fr[5]) + (fr[6] + fr[7])) + fr[8];
+        rb = ((fb[0] + fb[1]) + (fb[2] + fb[3])) + ((fb[4] + fb[5]) + (fb[6] + fb[7])) + fb[8];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = fr[i] + fb[i];
+        jx = ((f[1] + f[7]) + f[8]) - ((f[3] + f[5]) + f[4]);
+        jy = ((f[1] + f[3]) + f[2]) - ((f[5] + f[7]) + f[6]);
+        const float a = rr * P.inv_rho0_r, b = rb * P.inv_rho0_b;
+        const float inv = 1.0f / (a + b);
+        chr = a * inv;
+        chb = b * inv;
+        w[kChiR * kN] = chr;
+        w[kChiB * kN] = chb;
+        w[kPhi * kN] = fmaf(P.phip_r, rr, P.phip_b * rb);
+    }
+    __syncthreads();
+    // ---- grad rho^N on the smaller colour fraction, n-hat
+    float gx = 0.0f, gy = 0.0f;
+    if (inner(3)) {
+        const bool red_minor = chr <= 0.5f;
+        grad6(w + (red_minor ? kChiR : kChiB) * kN, gx, gy);
+        gx *= red_minor ? 2.0f : -2.0f;
+        gy *= red_minor ? 2.0f : -2.0f;
+        const float mag2 = fmaf(gx, gx, gy * gy);
+        const float inv = (mag2 >= kNormalTau * kNormalTau) ? rsqrtf(mag2) : 0.0f;
+        w[kNx * kN] = -gx * inv;
+        w[kNy * kN] = -gy * inv;
+    }
+    __syncthreads();
+    // ---- K, G, u
+    const float rho = rr + rb;
+    float Gx = 0.0f, Gy = 0.0f, ux = 0.0f, uy = 0.0f;
+    if (inner(4)) {
+        const float K = P.curvature_mode == 0 ? d_x(w + kNx * kN, 1.0f) + d_y(w + kNy * kN, -1.0f) : P.fixed_K;
+        const float hk = P.half_sigma * K;
+        Gx = fmaf(hk, gx, fmaf(rho, P.gacc_x, P.gvol_x));
+        Gy = fmaf(hk, gy, fmaf(rho, P.gacc_y, P.gvol_y));
+        ux = fmaf(0.5f, Gx, jx) / rho;
+        uy = fmaf(0.5f, Gy, jy) / rho;
+        w[kUx * kN] = ux;
+        w[kUy * kN] = uy;
+    }
+    __syncthreads();
+    // ---- the node's collision, recolour and store, or its fields
+    const size_t at = static_cast<size_t>(y) * nx;
+    if (MODE == Pass::Step) {
+        if (!own) return;
+        if (!isfinite(rho)) atomicOr(flag, 1u);
+        float dPx, dPy;
+        grad6(w + kPhi * kN, dPx, dPy);
+        const float divu = d_x(w + kUx * kN, -1.0f) + d_y(w + kUy * kN, -1.0f);
+        const float inv_rho = rcp(rho);
+        const float nu = P.visc_mode == 0
+                             ? fmaf(0.5f * (P.nu_r - P.nu_b), chr - chb, 0.5f * (P.nu_r + P.nu_b))
+                             : P.eta * inv_rho;
+        float fp[9];
+        collide_increment(f, rr, rb, rho, nu, ux, uy, Gx, Gy, dPx, dPy, divu, P, fp);
+        // recolour along e = grad rho^N / |grad rho^N| (Eq. eq_re_color; 0 below kNormalTau)
+        const float mag2 = fmaf(gx, gx, gy * gy);
+        const float inv = (mag2 >= kNormalTau * kNormalTau) ? rsqrtf(mag2) : 0.0f;
+        const float phim = fmaf(P.kphi_r, rr, P.kphi_b * rb) * inv_rho;
+        const float sg = P.beta * (rr * rb) * inv_rho * phim * inv;
+        store_recoloured_f32(dst + at, x, nodes, fp, rr, rb, inv_rho, sg * gx, sg * gy);
+    } else if (MODE == Pass::Fields) {
+        if (!own) return;
+        const size_t o = at + x;
+        if (fo.rho_r) fo.rho_r[o] = rr;
+        if (fo.rho_b) fo.rho_b[o] = rb;
+        if (fo.ux) fo.ux[o] = ux;
+        if (fo.uy) fo.uy[o] = uy;
+        if (fo.p) fo.p[o] = fmaf(P.cs2_r, rr, P.cs2_b * rb);
+    } else {
+        // FP64 partial diagnostics of the CTA (slot 4 is a maximum)
+        double v[kDiagSlots] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        if (own) {
+            if (isfinite(rho)) {
+                v[0] = rr;
+                v[1] = rb;
+                v[2] = jx;
+                v[3] = jy;
+                v[4] = static_cast<double>(ux) * ux + static_cast<double>(uy) * uy;
+            } else {
+                v[5] = 1.0;
+            }
+        }
+        __shared__ double red[H][kDiagSlots];
+#pragma unroll
+        for (int j = 0; j < kDiagSlots; ++j)
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                const double u = __shfl_down_sync(0xffffffffu, v[j], off);
+                v[j] = j == 4 ? fmax(v[j], u) : v[j] + u;
+            }
+        if (tx == 0)
+#pragma unroll
+            for (int j = 0; j < kDiagSlots; ++j) red[ty][j] = v[j];
+        __syncthreads();
+        if (threadIdx.x < kDiagSlots) {
+            double acc = 0.0;
+            for (int k = kEdge; k < H - kEdge; ++k)
+                acc = threadIdx.x == 4 ? fmax(acc, red[k][threadIdx.x]) : acc + red[k][threadIdx.x];
+            partials[(static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * kDiagSlots + threadIdx.x] = acc;
+        }
+    }
+}
+
+dim3 grid6(int nx, int ny, int H) {
+    const int tx = kX - 2 * kEdge, ty = H - 2 * kEdge;
+    return dim3(static_cast<unsigned>((nx + tx - 1) / tx), static_cast<unsigned>((ny + ty - 1) / ty));
+}
+
+// Window rows: 16 (two CTAs per SM) while that is at most two windows per SM, else 32.
+int rows6(int nx, int ny) {
+    const dim3 g = grid6(nx, ny, 16);
+    return static_cast<long>(g.x) * g.y <= 304 ? 16 : 32;
+}
+
+template <Pass MODE>
+cudaError_t launch6(const float* src, float* dst, const StepParams& P, FieldOut fo, unsigned* flag, double* partials,
+                    cudaStream_t s) {
+    const int H = rows6(P.nx, P.ny);
+    const dim3 g = grid6(P.nx, P.ny, H);
+    auto go = [&](auto k) { return launch_pdl(k, g, dim3(kX * H), 0, s, src, dst, P, fo, flag, partials); };
+    if (H == 16) return P.wall_y ? go(&k_order6<16, true, MODE>) : go(&k_order6<16, false, MODE>);
+    return P.wall_y ? go(&k_order6<32, true, MODE>) : go(&k_order6<32, false, MODE>);
+}
+
+}  // namespace
+
+cudaError_t launch_step6(const float* src, float* dst, const StepParams& P, unsigned* flag, cudaStream_t s) {
+    return launch6<Pass::Step>(src, dst, P, FieldOut{}, flag, nullptr, s);
+}
+cudaError_t launch_fields6(const float* src, const StepParams& P, FieldOut out, cudaStream_t s) {
+    return launch6<Pass::Fields>(src, nullptr, P, out, nullptr, nullptr, s);
+}
+int diag_blocks6(int nx, int ny) {
+    const dim3 g = grid6(nx, ny, rows6(nx, ny));
+    return static_cast<int>(g.x * g.y);
+}
+cudaError_t launch_diag6(const float* src, const StepParams& P, double* partials, cudaStream_t s) {
+    return launch6<Pass::Diag>(src, nullptr, P, FieldOut{}, nullptr, partials, s);
+}
+
+}  // namespace cmrt

@@ -1,15 +1,7 @@
-// Per-node plane passes (one thread per node, intermediate fields in global
-// planes) for FP32 storage: the step with App. B's order-6 gradient stencil,
-// and the discrete adjoint (reverse mode) of the step, arXiv 2005.04642,
-// Sec. 2, App. A, App. B.
-//
-// Order-6 step.  App. B's non-compact stencil d_a X = sum_N a_N sum_i w_i
-// X(r + N c_i) c_ia, (a_1, a_2, a_3) = (9/2, -9/10, 1/10), has radius 3; used
-// for grad rho^N and grad Phi' it widens the step's dependency radius from 3
-// to 5.  Rather than a second fused kernel with a wider halo and deeper
-// rings, the order-6 step runs as four passes over planes: moments, grad
-// rho^N, K / G / u (k_fwd_*, shared with the adjoint), then k_step_planes
-// (grad Phi', div u, collision, recolour, store).
+// The discrete adjoint (reverse mode) of the step, FP32 storage, arXiv
+// 2005.04642, Sec. 2, App. A, App. B: per-node passes over planes in memory (for
+// App. B's order-6 gradient stencil and mid-sized lattices), row wavefronts (large
+// lattices) and windows (small ones).
 //
 // The forward step maps the post-collision state P_{t-1} to P_t:
 //   f(t) = gather(P_{t-1})                       (streaming, Eq. equ_evolution)
@@ -37,6 +29,9 @@
 // per CTA (FP32 within a warp, FP64 from there) and accumulated across steps
 // in a per-CTA FP64 slot (no atomics: every launch of a pass uses the same
 // grid, and the slots are summed once at the end).
+#include <cooperative_groups.h>
+
+#include <algorithm>
 #include <atomic>
 #include <type_traits>
 
@@ -537,10 +532,13 @@ __device__ __forceinline__ void store_rev_collide(float* __restrict__ S, size_t 
 // The reverse collision pass: lam is the adjoint of the post-collision state P_t (18 planes).
 // F: the forward planes of post (the first kFwdPlanes planes of S, or those a
 // replayed step wrote); S: the adjoint's scratch planes.
-template <int ORDER, bool W>
+// PRE: lam is the adjoint of f(t + 1) in the public layout, read at the places
+// streaming takes P_t's populations to.
+template <int ORDER, bool W, bool PRE = false>
 __global__ void __launch_bounds__(kAT) k_rev_collide(const float* __restrict__ post, const float* __restrict__ lam,
                                                       const StepParams P, const float* __restrict__ F,
                                                       float* __restrict__ S, double* __restrict__ partials) {
+    pdl_begin();
     const int x = blockIdx.x * kAT + threadIdx.x, y = blockIdx.y;
     float acc[3] = {0.0f, 0.0f, 0.0f};  // beta, lambda3_r, lambda3_b
     if (x < P.nx) {
@@ -557,8 +555,15 @@ __global__ void __launch_bounds__(kAT) k_rev_collide(const float* __restrict__ p
         float lr[9], lb[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            lr[i] = lam[static_cast<size_t>(i) * L.n + o];
-            lb[i] = lam[static_cast<size_t>(9 + i) * L.n + o];
+            size_t at = o;
+            int li = i;
+            if (PRE) {
+                constexpr int R = reach<ORDER>();
+                if (W && L.mir[lcy(i) + R]) li = lopp(i);
+                else at = L.row[lcy(i) + R] + L.col[lcx(i) + R];
+            }
+            lr[i] = lam[static_cast<size_t>(li) * L.n + at];
+            lb[i] = lam[static_cast<size_t>(9 + li) * L.n + at];
         }
         RevCollide r;
         rev_collide_node(f, F[kRR * L.n + o], F[kRB * L.n + o], F[kUX * L.n + o], F[kUY * L.n + o],
@@ -935,6 +940,290 @@ __global__ void __launch_bounds__(kWin, 5) k_rev_tail(const StepParams P, const 
     }
 }
 
+// ----------------------------------------------------------------- reverse step by windows
+// One node per thread, a window of 32 x H nodes per CTA: the tail's stages with
+// a barrier each and no rows in series.  The row wavefront (k_rev_tail) is
+// bound by the latency of its row iterations on anything but a large lattice.
+// Two forms:
+// - split: the window form of the tail alone, after the collision pass; a
+//   window's own nodes are 24 x (H - 8).
+// - whole (tiny lattices, where launches count): the reverse collision too, its
+//   inputs loaded once and nothing but lambda written; 22 x (H - 10) own nodes,
+//   so that every collision runs 4 to 6 times.
+// The arithmetic is that of the plane passes, term by term in the same order.
+// VJP (cmrt_step_vjp): lam_out is the adjoint of f(t) (one halo node less), and
+// the whole form takes lam as the adjoint of f(t + 1), in the public layout.
+// first: the partial sums are written, not added to.
+constexpr int kRsX = 32;
+constexpr int rs_edge(bool vjp, bool split) { return (split ? 0 : 1) + (vjp ? 3 : 4); }
+// fields of the window in shared memory: Phi', u x, y, div-u-bar, K-bar; grad
+// rho^N-bar and grad Phi'-bar; and the adjoint's eleven populations and
+// densities, the first five in the place of the first five fields
+constexpr int kRsFields = 15;
+
+template <int H, bool W, bool VJP, bool SPLIT>
+__global__ void __launch_bounds__(kRsX * H, 2)
+    k_rev_small(const float* __restrict__ post, const float* __restrict__ lam, const StepParams P,
+                const float* __restrict__ F, const float* __restrict__ S, float* __restrict__ lam_out,
+                double* __restrict__ partials, bool first) {
+    pdl_begin();
+    constexpr int kN = kRsX * H, kEdge = rs_edge(VJP, SPLIT), kD = SPLIT ? 0 : 1;
+    extern __shared__ __align__(16) float rsm[];
+    const int tx = threadIdx.x % kRsX, ty = threadIdx.x / kRsX;
+    const int nx = P.nx, ny = P.ny;
+    const size_t n = static_cast<size_t>(nx) * ny;
+    const int xw = static_cast<int>(blockIdx.x) * (kRsX - 2 * kEdge) - kEdge + tx;
+    const int yw = static_cast<int>(blockIdx.y) * (H - 2 * kEdge) - kEdge + ty;
+    const int x = wrap_to(xw, nx), y = W ? yw : wrap_to(yw, ny);
+    const bool in = !W || (y >= 0 && y < ny);
+    auto inner = [&](int d) { return in && tx >= d && tx < kRsX - d && ty >= d && ty < H - d; };
+    const bool own = inner(kEdge) && xw < nx && yw < ny;
+    const bool low = W && y == 0, high = W && y == ny - 1;
+    float* w = rsm + kRsX + threadIdx.x;  // this node in a field of the window
+    constexpr int kPhi = 0, kU = 1, kV = 2, kDv = 3, kKb = 4, kGxb_ = 5, kGyb_ = 6, kPxb = 7, kPyb = 8;
+    auto lam_field = [](int j) { return j < 5 ? j : j + 4; };  // 0..8 links, 9 rho_R, 10 rho_B
+    // gradient of a field of the window: beyond a wall the node's own row, odd fields negated
+    const int up = high ? 0 : kRsX, dn = low ? 0 : -kRsX;
+    auto grad = [&](const float* a, float parity, float& gx, float& gy) {
+        const float pu = high ? parity : 1.0f, pd = low ? parity : 1.0f;
+        const float ne = pu * a[up + 1], nw = pu * a[up - 1], se = pd * a[dn + 1], sw = pd * a[dn - 1];
+        gx = ddx(a[1], a[-1], ne, nw, se, sw);
+        gy = ddy(pu * a[up], pd * a[dn], ne, nw, se, sw);
+    };
+    // its transpose (Nbh::gradT): a mirrored ghost row's reads are the wall row's own
+    auto gradT = [&](const float* a, bool xc, float parity) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            const int c = xc ? lcx(i) : lcy(i);
+            if (c == 0) continue;
+            const float k = 3.0f * lw(i) * float(c);
+            const int dx = -lcx(i), dy = -lcy(i);
+            if (!W || !((dy < 0 && low) || (dy > 0 && high))) acc = fmaf(k, a[dy * kRsX + dx], acc);
+            if (W && ((dy > 0 && low) || (dy < 0 && high))) acc = fmaf(parity * k, a[dx], acc);
+        }
+        return acc;
+    };
+
+    const unsigned o = in ? static_cast<unsigned>(y) * nx + x : 0u;
+    float rr = 1.0f, rb = 1.0f, ux = 0.0f, uy = 0.0f;
+    RevCollide r;
+    float gx = 0.0f, gy = 0.0f, K = 0.0f;
+    r.acc[0] = r.acc[1] = r.acc[2] = 0.0f;
+    if constexpr (SPLIT) {
+        if (in) {
+            w[kDv * kN] = __ldcg(S + kDIVUB * n + o);
+            w[kPxb * kN] = __ldcg(S + kDPXB * n + o);
+            w[kPyb * kN] = __ldcg(S + kDPYB * n + o);
+        }
+        if (inner(1)) {
+            ux = __ldcg(F + kUX * n + o);
+            uy = __ldcg(F + kUY * n + o);
+            rr = __ldcg(F + kRR * n + o);
+            rb = __ldcg(F + kRB * n + o);
+            gx = __ldcg(F + kGX * n + o);
+            gy = __ldcg(F + kGY * n + o);
+            K = __ldcg(F + kK * n + o);
+            r.uxb = __ldcg(S + kUXB * n + o);
+            r.uyb = __ldcg(S + kUYB * n + o);
+            r.Gxb = __ldcg(S + kGFXB * n + o);
+            r.Gyb = __ldcg(S + kGFYB * n + o);
+            r.gxb = __ldcg(S + kGXB * n + o);
+            r.gyb = __ldcg(S + kGYB * n + o);
+            r.rrb = __ldcg(S + kRRB * n + o);
+            r.rbb = __ldcg(S + kRBB * n + o);
+        }
+        if (inner(3)) {
+            r.rnb = __ldcg(S + kRNB * n + o);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) r.fbar[i] = __ldcg(S + static_cast<size_t>(kFB0 + i) * n + o);
+        }
+    } else {
+        if (in) {
+            ux = __ldcg(F + kUX * n + o);
+            uy = __ldcg(F + kUY * n + o);
+            w[kPhi * kN] = __ldcg(F + kPHIP * n + o);
+            w[kU * kN] = ux;
+            w[kV * kN] = uy;
+            rr = __ldcg(F + kRR * n + o);
+            rb = __ldcg(F + kRB * n + o);
+        }
+        __syncthreads();
+        // ---- reverse collision and recolour (k_rev_collide)
+        if (inner(1)) {
+            const unsigned xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+            const unsigned ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
+            // offset of the node (x + dx, y + dy), periodic
+            auto at = [&](int dx, int dy) {
+                return (dy > 0 ? yp : (dy < 0 ? ym : static_cast<unsigned>(y))) * nx +
+                       (dx > 0 ? xp : (dx < 0 ? xm : static_cast<unsigned>(x)));
+            };
+            float f[9], lr[9], lb[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                unsigned src = at(-lcx(i), -lcy(i));
+                int li = i;
+                if (W && ((lcy(i) > 0 && low) || (lcy(i) < 0 && high))) {
+                    li = lopp(i);
+                    src = o;
+                }
+                f[i] = __ldcg(post + static_cast<size_t>(li) * n + src) + __ldcg(post + static_cast<size_t>(9 + li) * n + src);
+                unsigned dst = o;
+                int lj = i;
+                if (VJP) {
+                    dst = at(lcx(i), lcy(i));
+                    if (W && ((lcy(i) > 0 && high) || (lcy(i) < 0 && low))) {
+                        lj = lopp(i);
+                        dst = o;
+                    }
+                }
+                lr[i] = __ldcg(lam + static_cast<size_t>(lj) * n + dst);
+                lb[i] = __ldcg(lam + static_cast<size_t>(9 + lj) * n + dst);
+            }
+            float dPx, dPy, dux, duy, t0, t1;
+            grad(w + kPhi * kN, 1.0f, dPx, dPy);
+            grad(w + kU * kN, -1.0f, dux, t0);
+            grad(w + kV * kN, -1.0f, t1, duy);
+            gx = __ldcg(F + kGX * n + o);
+            gy = __ldcg(F + kGY * n + o);
+            K = __ldcg(F + kK * n + o);
+            rev_collide_node(f, rr, rb, ux, uy, __ldcg(F + kGFX * n + o), __ldcg(F + kGFY * n + o), gx, gy, __ldcg(F + kCHR * n + o) - __ldcg(F + kCHB * n + o),
+                             dPx, dPy, dux + duy, lr, lb, P, r);
+            w[kDv * kN] = r.divub;
+            w[kPxb * kN] = r.dPxb;
+            w[kPyb * kN] = r.dPyb;
+        }
+    }
+    __syncthreads();
+    // ---- R2: reverse of div u, u = (j + G/2) / rho and G (k_rev_force)
+    float ps = 0.0f, pgx = 0.0f, pgy = 0.0f;
+    float jxb = 0.0f, jyb = 0.0f;
+    if (inner(kD + 1)) {
+        const float uxt = r.uxb + gradT(w + kDv * kN, true, -1.0f);
+        const float uyt = r.uyb + gradT(w + kDv * kN, false, -1.0f);
+        const float rho = rr + rb;
+        const float ir = 1.0f / rho;
+        const float Gxt = fmaf(0.5f * ir, uxt, r.Gxb);
+        const float Gyt = fmaf(0.5f * ir, uyt, r.Gyb);
+        const float rhob = -(ux * uxt + uy * uyt) * ir + Gxt * P.gacc_x + Gyt * P.gacc_y;
+        const float gG = fmaf(Gxt, gx, Gyt * gy);
+        jxb = uxt * ir;
+        jyb = uyt * ir;
+        w[kKb * kN] = P.half_sigma * gG;
+        r.gxb += P.half_sigma * K * Gxt;
+        r.gyb += P.half_sigma * K * Gyt;
+        r.rrb += rhob;
+        r.rbb += rhob;
+        if (own) {
+            ps = 0.5f * K * gG;
+            pgx = rho * Gxt;
+            pgy = rho * Gyt;
+        }
+    }
+    __syncthreads();
+    // ---- R3: reverse of K = div n-hat and of the normal (k_rev_normal)
+    if (inner(kD + 2)) {
+        if (P.curvature_mode == 0) {
+            const float nxb = gradT(w + kKb * kN, true, 1.0f);
+            const float nyb = gradT(w + kKb * kN, false, -1.0f);
+            float ox, oy;
+            normalise_T(gx, gy, nxb, nyb, ox, oy);
+            r.gxb -= ox;
+            r.gyb -= oy;
+        }
+    }
+    w[kGxb_ * kN] = r.gxb;
+    w[kGyb_ * kN] = r.gyb;
+    __syncthreads();
+    // ---- R4: reverse of the gradients, rho^N, Phi' and the moments (k_rev_moments)
+    if (inner(kD + 3)) {
+        float rnb = r.rnb;
+        rnb += gradT(w + kGxb_ * kN, true, 1.0f) + gradT(w + kGyb_ * kN, false, 1.0f);
+        const float phb = gradT(w + kPxb * kN, true, 1.0f) + gradT(w + kPyb * kN, false, 1.0f);
+        const float a = rr * P.inv_rho0_r, b = rb * P.inv_rho0_b;
+        const float iden = 1.0f / ((a + b) * (a + b));
+        r.rrb += fmaf(rnb * 2.0f * b * iden, P.inv_rho0_r, phb * P.phip_r);
+        r.rbb += fmaf(rnb * -2.0f * a * iden, P.inv_rho0_b, phb * P.phip_b);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            if (lcx(i)) r.fbar[i] += float(lcx(i)) * jxb;
+            if (lcy(i)) r.fbar[i] += float(lcy(i)) * jyb;
+        }
+    }
+    // ---- R5: lambda (k_rev_gather / k_rev_expand)
+    if (VJP) {
+        if (own) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                lam_out[static_cast<size_t>(i) * n + o] = r.fbar[i] + r.rrb;
+                lam_out[static_cast<size_t>(9 + i) * n + o] = r.fbar[i] + r.rbb;
+            }
+        }
+    } else {
+        if (inner(kD + 3)) {  // the first five fields are done with; the others R4 read
+#pragma unroll
+            for (int i = 0; i < 9; ++i) w[lam_field(i) * kN] = r.fbar[i];
+            w[lam_field(9) * kN] = r.rrb;
+            w[lam_field(10) * kN] = r.rbb;
+        }
+        __syncthreads();
+        if (own) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const bool wall = W && ((lcy(i) > 0 && high) || (lcy(i) < 0 && low));
+                const int li = wall ? lopp(i) : i;
+                const float* a = w + (wall ? 0 : lcy(i) * kRsX + lcx(i));
+                const float common = a[lam_field(li) * kN];
+                lam_out[static_cast<size_t>(i) * n + o] = common + a[lam_field(9) * kN];
+                lam_out[static_cast<size_t>(9 + i) * n + o] = common + a[lam_field(10) * kN];
+            }
+        }
+    }
+    // ---- parameter gradients of the own nodes: beta and lambda_3 as add_partials
+    // (FP32 within a warp), sigma and g_acc in FP64 from each node's term on, by
+    // three warps, a lane per column (a warp's FP64 add takes the SM 16 cycles)
+    __shared__ double red[H][3], col[3];
+    if (!SPLIT) {
+        float q[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            q[j] = own ? r.acc[j] : 0.0f;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) q[j] += __shfl_down_sync(0xffffffffu, q[j], off);
+        }
+        if (tx == 0) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) red[ty][j] = static_cast<double>(q[j]);
+        }
+    }
+    // the fields grad rho^N-bar and grad Phi'-bar are done with (not read since R4)
+    if (VJP) __syncthreads();
+    w[kGxb_ * kN] = ps;
+    w[kGyb_ * kN] = pgx;
+    w[kPxb * kN] = pgy;
+    __syncthreads();
+    if (ty < 3) {
+        const float* term = rsm + kRsX + (kGxb_ + ty) * kN + tx;
+        double v = 0.0;
+        for (int k = kEdge; k < H - kEdge; ++k) v += static_cast<double>(term[k * kRsX]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        if (tx == 0) col[ty] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < kAdjSlots) {
+        // slots: sigma, beta, lambda3_r, lambda3_b, g_acc_x, g_acc_y
+        const int j = threadIdx.x;
+        double a = 0.0;
+        if (!SPLIT && j >= 1 && j <= 3)
+            for (int k = kEdge; k < H - kEdge; ++k) a += red[k][j - 1];
+        else if (j == 0 || j == 4 || j == 5)
+            a = col[j == 0 ? 0 : j - 3];
+        double* slot = partials + (static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * kAdjSlots + threadIdx.x;
+        *slot = first ? a : *slot + a;
+    }
+}
+
 // rows per CTA of the fused tail: enough CTAs for two waves of 152 SMs where
 // the lattice allows, at most 64 rows (8 fill iterations per segment)
 int tail_rows(int nx, int ny) {
@@ -1226,125 +1515,40 @@ __global__ void __launch_bounds__(kAT) k_init_T(const float* __restrict__ pre0, 
     grad[o] = 0.5f * (rrb / P.inv_rho0_r - rbb / P.inv_rho0_b);
 }
 
-// ----------------------------------------------------------------- order-6 step and its outputs
-// The rest of one step after k_fwd_*: grad Phi' (order of P.stencil_order),
-// div u, collision in moment space, recolour and store of P_t (FP32 layout).
-template <int ORDER, bool W>
-__global__ void __launch_bounds__(kAT) k_step_planes(const float* __restrict__ post, float* __restrict__ dst,
-                                                      const StepParams P, const float* __restrict__ S,
-                                                      unsigned* __restrict__ flag) {
-    const int x = blockIdx.x * kAT + threadIdx.x, y = blockIdx.y;
-    if (x >= P.nx) return;
-    const Nbh<reach<ORDER>(), W> L(P, x, y);
-    const size_t o = L.o;
-    float fr[9], fb[9], f[9];
-    L.gather(post, fr, fb);
-    const float rr = sum9f(fr), rb = sum9f(fb);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) f[i] = fr[i] + fb[i];
-    const float rho = rr + rb;
-    if (!isfinite(rho)) atomicOr(flag, 1u);
-    float dPx, dPy, dux, duy, t0, t1;
-    L.template grad<ORDER>(S + kPHIP * L.n, 1.0f, dPx, dPy);
-    L.template grad<2>(S + kUX * L.n, -1.0f, dux, t0);
-    L.template grad<2>(S + kUY * L.n, -1.0f, t1, duy);
-    const float inv_rho = rcp(rho);
-    float nu;
-    if (P.visc_mode == 0) {
-        const float rn = S[kCHR * L.n + o] - S[kCHB * L.n + o];
-        nu = fmaf(0.5f * (P.nu_r - P.nu_b), rn, 0.5f * (P.nu_r + P.nu_b));
-    } else {
-        nu = P.eta * inv_rho;
-    }
-    float fp[9];
-    collide_increment(f, rr, rb, rho, nu, S[kUX * L.n + o], S[kUY * L.n + o], S[kGFX * L.n + o],
-                      S[kGFY * L.n + o], dPx, dPy, dux + duy, P, fp);
-    // recolour along e = grad rho^N / |grad rho^N| (Eq. eq_re_color; 0 below kNormalTau)
-    const float gx = S[kGX * L.n + o], gy = S[kGY * L.n + o];
-    const float mag2 = fmaf(gx, gx, gy * gy);
-    const float inv = (mag2 >= kNormalTau * kNormalTau) ? rsqrtf(mag2) : 0.0f;
-    const float phim = fmaf(P.kphi_r, rr, P.kphi_b * rb) * inv_rho;
-    const float sg = P.beta * (rr * rb) * inv_rho * phim * inv;
-    store_recoloured_f32(dst + L.row[reach<ORDER>()], x, L.n, fp, rr, rb, inv_rho, sg * gx, sg * gy);
-}
-
-__global__ void __launch_bounds__(kAT) k_fields_planes(const StepParams P, const float* __restrict__ S,
-                                                        FieldOut fo) {
-    const int x = blockIdx.x * kAT + threadIdx.x, y = blockIdx.y;
-    if (x >= P.nx) return;
-    const Own L(P, x, y);
-    const size_t o = L.o;
-    const float rr = S[kRR * L.n + o], rb = S[kRB * L.n + o];
-    if (fo.rho_r) fo.rho_r[o] = rr;
-    if (fo.rho_b) fo.rho_b[o] = rb;
-    if (fo.ux) fo.ux[o] = S[kUX * L.n + o];
-    if (fo.uy) fo.uy[o] = S[kUY * L.n + o];
-    if (fo.p) fo.p[o] = fmaf(P.cs2_r, rr, P.cs2_b * rb);
-}
-
-// FP64 per-CTA partial diagnostics, partials[block][kDiagSlots] (slot 4 is a maximum)
-__global__ void __launch_bounds__(kAT) k_diag_planes(const StepParams P, const float* __restrict__ S,
-                                                      double* __restrict__ partials) {
-    const int x = blockIdx.x * kAT + threadIdx.x, y = blockIdx.y;
-    double v[kDiagSlots] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (x < P.nx) {
-        const Own L(P, x, y);
-        const size_t o = L.o;
-        const float rr = S[kRR * L.n + o], rb = S[kRB * L.n + o];
-        if (isfinite(rr + rb)) {
-            const double ux = S[kUX * L.n + o], uy = S[kUY * L.n + o];
-            v[0] = rr;
-            v[1] = rb;
-            v[2] = S[kJX * L.n + o];
-            v[3] = S[kJY * L.n + o];
-            v[4] = ux * ux + uy * uy;
-        } else {
-            v[5] = 1.0;
-        }
-    }
-    __shared__ double red[kAT / 32][kDiagSlots];
-#pragma unroll
-    for (int j = 0; j < kDiagSlots; ++j)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const double w = __shfl_down_sync(0xffffffffu, v[j], off);
-            v[j] = j == 4 ? fmax(v[j], w) : v[j] + w;
-        }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0)
-#pragma unroll
-        for (int j = 0; j < kDiagSlots; ++j) red[warp][j] = v[j];
+// The slots of all CTAs, summed: one cluster of kRedCtas CTAs, each over its
+// share of the rows (a warp reads four rows of eight slots at once), then the
+// first over the shares through distributed shared memory.  A fixed order, so
+// the sums are reproducible.  One CTA of 128 threads took 208 us for the 32768
+// rows of a 2048^2 lattice and 26 us for 3072, a load latency per 128 rows; this
+// takes 9 and 4 us.
+constexpr int kRedCtas = 8, kRedThreads = 512;
+__global__ void __cluster_dims__(kRedCtas, 1, 1) __launch_bounds__(kRedThreads)
+    k_adj_reduce(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
+    constexpr int kWarps = kRedThreads / 32, kRows = kRedThreads / kAdjSlots;
+    static_assert(kAdjSlots == 8, "a warp reads four rows");
+    __shared__ double red[kWarps][kAdjSlots];
+    __shared__ double mine[kAdjSlots];
+    const int t = threadIdx.x, slot = t % kAdjSlots;
+    double v = 0.0;
+    for (int b = blockIdx.x * kRows + t / kAdjSlots; b < nblocks; b += kRedCtas * kRows)
+        v += partials[static_cast<size_t>(b) * kAdjSlots + slot];
+    v += __shfl_down_sync(0xffffffffu, v, 16);
+    v += __shfl_down_sync(0xffffffffu, v, 8);
+    if ((t & 31) < kAdjSlots) red[t >> 5][slot] = v;
     __syncthreads();
-    if (threadIdx.x < kDiagSlots) {
-        double acc = red[0][threadIdx.x];
-        for (int w = 1; w < kAT / 32; ++w)
-            acc = threadIdx.x == 4 ? fmax(acc, red[w][threadIdx.x]) : acc + red[w][threadIdx.x];
-        partials[(static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * kDiagSlots + threadIdx.x] = acc;
+    if (t < kAdjSlots) {
+        double a = 0.0;
+        for (int w = 0; w < kWarps; ++w) a += red[w][t];
+        mine[t] = a;
     }
-}
-
-__global__ void k_adj_reduce(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {
-    __shared__ double red[kAT / 32][kAdjSlots];
-    double v[kAdjSlots];
-#pragma unroll
-    for (int j = 0; j < kAdjSlots; ++j) v[j] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-        for (int j = 0; j < kAdjSlots; ++j) v[j] += partials[static_cast<size_t>(b) * kAdjSlots + j];
-#pragma unroll
-    for (int j = 0; j < kAdjSlots; ++j)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v[j] += __shfl_down_sync(0xffffffffu, v[j], off);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0)
-#pragma unroll
-        for (int j = 0; j < kAdjSlots; ++j) red[warp][j] = v[j];
-    __syncthreads();
-    if (threadIdx.x < kAdjSlots) {
-        double acc = 0.0;
-        for (int w = 0; w < kAT / 32; ++w) acc += red[w][threadIdx.x];
-        out[threadIdx.x] = acc;
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    if (blockIdx.x == 0 && t < kAdjSlots) {
+        double a = 0.0;
+        for (int c = 0; c < kRedCtas; ++c) a += *cluster.map_shared_rank(&mine[t], c);
+        out[t] = a;
     }
+    cluster.sync();  // the shares outlive the read
 }
 
 dim3 adj_grid(const StepParams& P) { return dim3(static_cast<unsigned>((P.nx + kAT - 1) / kAT), P.ny, 1); }
@@ -1372,6 +1576,68 @@ void forward_planes(const float* post, const StepParams& P, float* S, cudaStream
     k_fwd_force<W><<<g, kAT, 0, s>>>(P, S);
 }
 
+// The reverse step by windows: compact stencil, not with the plane passes asked
+// for, up to 400 000 nodes in an adjoint sweep, up to 900 000 in a step VJP
+// (whose alternative is the plane passes or recomputes the forward fields in a
+// row wavefront); the whole form up to 9000.  Measured, us per step of an
+// adjoint call with checkpoints (its forward run and replay included), before
+// -> by windows: 64^2 26.7 -> 9.8 (whole; split 11.0), 128^2 30.9 -> 13.6
+// (split; whole 14.2), 256^2 42.6 -> 23.2, 320^2 45.1 -> 30.2, 512^2 87.8 -> 62.7;
+// 640^2 91.8 against 97.2 and 2048^2 676 against 837, so not there.  Step VJP
+// (device and host): 256^2 88 -> 56 us, 1024 x 384 165 -> 105, 640^2 147 -> 111,
+// 1024^2 207 either way.
+constexpr long kRevSweepNodes = 400000, kRevVjpNodes = 900000, kRevWholeNodes = 9000;
+long lattice_nodes(const StepParams& P) { return static_cast<long>(P.nx) * P.ny; }
+bool rev_small(const StepParams& P, bool vjp) {
+    return P.stencil_order == 2 && P.adjoint_fused != 2 && lattice_nodes(P) <= (vjp ? kRevVjpNodes : kRevSweepNodes);
+}
+bool rev_whole(const StepParams& P) { return lattice_nodes(P) <= kRevWholeNodes; }
+dim3 rev_small_grid(const StepParams& P, int H, bool vjp, bool split) {
+    const int e = rs_edge(vjp, split), tx = kRsX - 2 * e, ty = H - 2 * e;
+    return dim3(static_cast<unsigned>((P.nx + tx - 1) / tx), static_cast<unsigned>((P.ny + ty - 1) / ty));
+}
+// Window rows: 12 where that is little more than one window per SM (64^2 whole
+// 9.8 us against 11.3 with 16 rows, 128^2 split 13.6 against 14.5), else 16
+// (256^2 23.2 against 25.5 with 12 and 23.9 with 32; 512^2 62.7, 73.9, 67.1).
+int rev_small_rows(const StepParams& P, bool vjp, bool split) {
+    const dim3 g = rev_small_grid(P, 12, vjp, split);
+    return static_cast<long>(g.x) * g.y <= 200 ? 12 : 16;
+}
+
+template <int H, bool W, bool VJP, bool SPLIT>
+cudaError_t launch_rev_small_h(const float* post, const float* lam, const StepParams& P, const float* F, const float* S,
+                               float* lam_out, double* partials, bool first, cudaStream_t s) {
+    constexpr int smem = (kRsFields * kRsX * H + 2 * kRsX) * 4;
+    static std::atomic<unsigned long long> configured{0};  // the shared-memory opt-in, once per device (any thread)
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(configured.load() & bit)) {
+        e = cudaFuncSetAttribute(k_rev_small<H, W, VJP, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        configured.fetch_or(bit);
+    }
+    return launch_pdl(k_rev_small<H, W, VJP, SPLIT>, rev_small_grid(P, H, VJP, SPLIT), dim3(kRsX * H), smem, s, post, lam,
+                      P, F, S, lam_out, partials, first);
+}
+
+// One reverse step by windows, F the forward fields of post.
+template <bool W, bool VJP>
+cudaError_t launch_rev_small(const float* post, const float* lam, const StepParams& P, const float* F, float* S,
+                             float* lam_out, double* partials, bool first, cudaStream_t s) {
+    auto go = [&](auto split) {
+        constexpr bool SPLIT = decltype(split)::value;
+        if (rev_small_rows(P, VJP, SPLIT) == 12)
+            return launch_rev_small_h<12, W, VJP, SPLIT>(post, lam, P, F, S, lam_out, partials, first, s);
+        return launch_rev_small_h<16, W, VJP, SPLIT>(post, lam, P, F, S, lam_out, partials, first, s);
+    };
+    if (rev_whole(P)) return go(std::false_type{});
+    const dim3 g(static_cast<unsigned>((P.nx + kAT - 1) / kAT), P.ny, 1);
+    const cudaError_t e = launch_pdl(k_rev_collide<2, W, VJP>, g, dim3(kAT), 0, s, post, lam, P, F, S, partials);
+    return e != cudaSuccess ? e : go(std::true_type{});
+}
+
 // One adjoint step: `lam_out` is lambda of P_{t-1} (transposed gather) or,
 // with EXPAND, dJ/df(t) in the public layout.  With the compact stencil on a
 // large enough lattice it is three launches (k_fwd_head: the forward fields;
@@ -1381,6 +1647,13 @@ template <int O, bool W, bool EXPAND>
 cudaError_t reverse_step(const float* post, const float* lam_post, const StepParams& P, float* S, double* partials,
                          float* lam_out, cudaStream_t s, const float* fwd) {
     const dim3 g = adj_grid(P);
+    if (O == 2 && !EXPAND && rev_small(P, false)) {
+        if (!fwd) {
+            const cudaError_t e = launch_fwd_fields(post, P, S, s);
+            if (e != cudaSuccess) return e;
+        }
+        return launch_rev_small<W, false>(post, lam_post, P, fwd ? fwd : S, S, lam_out, partials, false, s);
+    }
     if (O == 2 && use_fused(P)) {
         // the forward fields of post: written by the replayed step, or recomputed here
         const float* F = fwd;
@@ -1405,41 +1678,30 @@ cudaError_t reverse_step(const float* post, const float* lam_post, const StepPar
 }  // namespace
 
 int adj_blocks(int nx, int ny) {
-    // per-CTA partial-sum slots: the larger of the plane passes' grid and the fused tail's
+    // per-CTA partial-sum slots: the larger of the plane passes' grid, the fused tail's and the small-lattice kernel's
     const int planes = ((nx + kAT - 1) / kAT) * ny;
     const int rows = tail_rows(nx, ny);
     const int tail = ((nx + kTileX - 1) / kTileX) * ((ny + rows - 1) / rows);
-    return planes > tail ? planes : tail;
+    int most = std::max(planes, tail);
+    StepParams P{};
+    P.nx = nx;
+    P.ny = ny;
+    if (lattice_nodes(P) <= kRevVjpNodes)
+        for (const bool vjp : {false, true}) {
+            const bool split = !rev_whole(P);
+            const dim3 g = rev_small_grid(P, rev_small_rows(P, vjp, split), vjp, split);
+            most = std::max(most, static_cast<int>(g.x * g.y));
+        }
+    return most;
 }
 
-cudaError_t launch_step_planes(const float* post, float* dst, const StepParams& P, float* scratch, unsigned* flag,
-                               cudaStream_t s) {
-    dispatch(P, [&](auto o, auto w) {
-        forward_planes<decltype(o)::value, decltype(w)::value>(post, P, scratch, s);
-        k_step_planes<decltype(o)::value, decltype(w)::value><<<adj_grid(P), kAT, 0, s>>>(post, dst, P, scratch, flag);
-    });
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fields_planes(const float* post, const StepParams& P, float* scratch, FieldOut out,
-                                 cudaStream_t s) {
-    dispatch(P, [&](auto o, auto w) { forward_planes<decltype(o)::value, decltype(w)::value>(post, P, scratch, s); });
-    k_fields_planes<<<adj_grid(P), kAT, 0, s>>>(P, scratch, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_diag_planes(const float* post, const StepParams& P, float* scratch, double* partials,
-                               cudaStream_t s) {
-    dispatch(P, [&](auto o, auto w) { forward_planes<decltype(o)::value, decltype(w)::value>(post, P, scratch, s); });
-    k_diag_planes<<<adj_grid(P), kAT, 0, s>>>(P, scratch, partials);
-    return cudaGetLastError();
-}
-
-bool adj_fused(const StepParams& P) { return P.stencil_order == 2 && use_fused(P); }
+bool adj_fused(const StepParams& P) { return P.stencil_order == 2 && (use_fused(P) || rev_small(P, false)); }
 bool adj_fields_usable(const StepParams& P) { return P.stencil_order == 2 && P.adjoint_fused != 2; }
 
-int adj_launches_per_step(const StepParams& P) {
-    if (adj_fused(P)) return 3;  // fused forward fields, collision pass, fused tail
+int adj_launches_per_step(const StepParams& P, bool vjp) {
+    // forward fields, (collision pass,) the reverse step by windows
+    if (rev_small(P, vjp)) return rev_whole(P) ? 2 : 3;
+    if (P.stencil_order == 2 && use_fused(P)) return 3;  // fused forward fields, collision pass, fused tail
     return P.curvature_mode == 0 ? 8 : 7;
 }
 
@@ -1452,6 +1714,20 @@ cudaError_t launch_adjoint_step(const float* post, const float* lam_post, const 
                                                                        s, fwd);
     });
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+bool adj_vjp_small(const StepParams& P) { return rev_small(P, true); }
+int adj_vjp_small_blocks(const StepParams& P) {
+    const dim3 g = rev_small_grid(P, rev_small_rows(P, true, false), true, false);
+    return rev_whole(P) ? static_cast<int>(g.x * g.y) : adj_blocks(P.nx, P.ny);
+}
+
+cudaError_t launch_vjp_small(const float* post, const float* lam_next, const StepParams& P, float* scratch,
+                             double* partials, float* lam, cudaStream_t s) {
+    const cudaError_t e = launch_fwd_fields(post, P, scratch, s);
+    if (e != cudaSuccess) return e;
+    return P.wall_y ? launch_rev_small<true, true>(post, lam_next, P, scratch, scratch, lam, partials, rev_whole(P), s)
+                    : launch_rev_small<false, true>(post, lam_next, P, scratch, scratch, lam, partials, rev_whole(P), s);
 }
 
 cudaError_t launch_adjoint_step_pre(const float* post, const float* lam_post, const StepParams& P, float* scratch,
@@ -1484,7 +1760,7 @@ cudaError_t launch_adjoint_init(const float* pre0, const float* lam_pre0, const 
 }
 
 cudaError_t launch_adjoint_reduce(const double* partials, int nblocks, double* out, cudaStream_t s) {
-    k_adj_reduce<<<1, kAT, 0, s>>>(partials, nblocks, out);
+    k_adj_reduce<<<kRedCtas, kRedThreads, 0, s>>>(partials, nblocks, out);
     return cudaGetLastError();
 }
 

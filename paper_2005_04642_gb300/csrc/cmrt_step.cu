@@ -97,6 +97,12 @@ cudaError_t launch_step_fields(const float* src, float* dst, const StepParams& P
     return launch_march<MarchF32<kWin>, Pass::StepFields>(src, dst, P, rows, fo, flag, nullptr, s);
 }
 
+cudaError_t launch_fwd_fields(const float* src, const StepParams& P, float* fwd, cudaStream_t s) {
+    FieldOut fo{};
+    fo.fwd = fwd;
+    return launch_small_any<MarchF32<kWin>, Pass::FwdFields>(src, nullptr, P, fo, nullptr, s);
+}
+
 cudaError_t launch_fields(const void* src, const StepParams& P, int rows, FieldOut out, cudaStream_t s) {
     if (P.precision != kPrecF32) return launch_fields16(src, P, rows, out, s);
     return launch_march<MarchF32<kWin>, Pass::Fields>(src, nullptr, P, rows, out, nullptr, nullptr, s);

@@ -1,0 +1,104 @@
+"""The forms of one pass that a size rule chooses between: windows of one node
+per thread (small lattices, App. B's stencil, the reverse step) and the row
+march (large lattices, batches), at the edges of their tiles.
+
+Two forms of the forward step compute the same expressions, so their
+populations must be equal bit for bit; the reverse step's forms sum in another
+order and are held to the tolerance of the tests that compare its other forms
+(1e-5 of each gradient).  Forms that no smaller lattice reaches are compared
+with the FP64 oracle at the parity tests' bar for a few steps (2e-6 of the
+largest population)."""
+import numpy as np
+import pytest
+
+from oracle import cmrt_oracle as O
+from paper_2005_04642_gb300 import inputs as I
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU machines too
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2005_04642_gb300 import cmrt as cm  # noqa: E402
+
+cm.load()
+
+
+def _setup(nx, ny, wall, **kw):
+    d = I.base_params(nx, ny, wall_y=wall, g_acc=(1e-5, -2e-5), **kw)
+    rn, u = I.random_state_fields(nx, ny, seed=nx + 3 * ny, amplitude=0.02)
+    return d, rn.astype(np.float32), u.astype(np.float32)
+
+
+# own columns of a window: 26 or 24 (one node per thread), 88 or 120 (march);
+# own rows 2, 4, 8, 10; widths that copy 16 bytes at a time and that do not
+SHAPES = [(24, 8), (25, 9), (26, 10), (27, 11), (53, 21), (88, 40), (89, 5), (176, 23), (120, 64), (121, 12),
+          (248, 31), (512, 66)]
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2], ids=["fp32", "bf16", "fp16"])
+@pytest.mark.parametrize("wall", [False, True], ids=["periodic", "walls"])
+def test_windows_and_march_give_the_same_bits(precision, wall):
+    """A lattice of this size steps by windows; a batch member by the march."""
+    members = [_setup(nx, ny, wall, precision=precision) for nx, ny in SHAPES]
+    for pick in (slice(None), slice(5, 8), slice(8, 11)):  # 88- and 120-column strips
+        b = cm.Batch(members[pick])
+        b.step(3)
+        for k, m in enumerate(members[pick]):
+            lat = cm.Lattice(*m)
+            lat.step(3)
+            assert torch.equal(b.member(k).populations(), lat.populations()), (m[0]["nx"], m[0]["ny"])
+            lat.close()
+        b.close()
+
+
+@pytest.mark.parametrize("nx,ny,wall,order", [(1024, 600, False, 2), (1024, 600, True, 2), (1001, 701, False, 2),
+                                              (1001, 701, True, 2), (230, 400, False, 6), (230, 401, True, 6)])
+def test_forms_of_larger_lattices_match_oracle(nx, ny, wall, order):
+    """The march of a single lattice (16-byte and 4-byte copies) and the taller
+    windows of App. B's stencil."""
+    d = I.base_params(nx, ny, wall_y=wall, g_acc=(1e-5, -2e-5), stencil_order=order)
+    rn = I.drops_field(nx, ny, [(0.3 * nx + 0.3, 0.45 * ny - 0.2), (1.5, 0.6 * ny + 0.4)], [0.2 * min(nx, ny), 40.0],
+                       periodic_y=not wall)
+    u = I.velocity_noise(nx, ny, 0.01, 7)
+    lat = cm.Lattice(d, rn.astype(np.float32), u.astype(np.float32))
+    lat.step(3)
+    got = lat.populations().double().cpu().numpy()
+    p = O.Params(**d)
+    R, B = O.init_state(rn.astype(np.float32).astype(np.float64), *u.astype(np.float32).astype(np.float64), p)
+    R, B = O.run(R, B, p, 3)
+    ref = np.stack([R, B])
+    assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max()
+    lat.close()
+
+
+@pytest.mark.parametrize("nx,ny,wall", [(64, 64, False), (23, 300, True), (100, 101, False), (131, 90, True),
+                                        (300, 260, False), (512, 400, True)])
+def test_reverse_step_by_windows_matches_plane_passes(nx, ny, wall):
+    """Sweeps whose lattices take the whole form (up to 9000 nodes) and the split
+    one with 12 and 16 window rows, with recomputed and with written forward
+    fields, and the step VJP, also in place."""
+    rn = I.drops_field(nx, ny, [(0.5 * nx + 0.3, 0.5 * ny - 0.2)], [0.25 * min(nx, ny)], periodic_y=not wall)
+    target = I.drops_field(nx, ny, [(0.5 * nx + 1.3, 0.5 * ny + 0.3)], [0.25 * min(nx, ny)], periodic_y=not wall)
+    u = I.velocity_noise(nx, ny, 0.01, 5).astype(np.float32)
+    lam = torch.from_numpy(np.random.default_rng(6).standard_normal((2, 9, ny, nx)).astype(np.float32)).cuda()
+    outs = []
+    for fused in (0, 2):
+        d = I.base_params(nx, ny, wall_y=wall, g_acc=(1e-5, -2e-5), adjoint_fused=fused)
+        lat = cm.Lattice(d, rn.astype(np.float32), u)
+        v, gv = lat.step_vjp(lam)
+        if fused == 0:
+            same = lam.clone()
+            g2 = cm.cmrt_step_vjp(lat.ctx, same.data_ptr(), same.data_ptr())
+            assert torch.equal(same, v) and g2 == gv
+        J, g, grn = lat.adjoint(6, target.astype(np.float32), ckpt_every=4, want_rho_n0=True)
+        outs.append((J, list(g.values()), gv, grn.double(), v.double()))
+        lat.close()
+    (J0, g0, gv0, r0, v0), (J2, g2, gv2, r2, v2) = outs
+    assert J0 == J2
+    for a, b in ((g0, g2), (gv0, gv2)):
+        top = max(abs(x) for x in b)
+        assert all(abs(x - y) <= 1e-5 * abs(y) + 1e-7 * top for x, y in zip(a, b)), (a, b)
+    assert (r0 - r2).abs().max() <= 1e-5 * r2.abs().max()
+    assert (v0 - v2).abs().max() <= 1e-5 * v2.abs().max()
