@@ -234,7 +234,8 @@ struct Layout16 {
         weights(rr, rb, inv_rho, nfree, P, wa, wd);
         const float2 refa = __fmul2_rn(rho2, wa);  // the decoder's reference pairs
         const float2 refd = __fmul2_rn(rho2, wd);
-        const float2 a2 = make_float2(rr * inv_rho * S, rb * inv_rho * S), mrho = make_float2(-rr * S, -rb * S);
+        const float ar = rr * inv_rho * S, ab = rb * inv_rho * S;
+        const float2 mrho = make_float2(-rr * S, -rb * S);
         const float2 mS = make_float2(-S, -S), pS = make_float2(S, S), m1 = make_float2(-1.0f, -1.0f);
         const float2 un2 = make_float2(P.dev_unscale, P.dev_unscale);
         // The rest populations are what is left of rho_R and rho_B after the
@@ -244,7 +245,8 @@ struct Layout16 {
         float2 sum = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int i = 1; i < 9; ++i) {
-            float2 C = __ffma2_rn(a2, make_float2(fp[i], fp[i]), make_float2(seg[i], -seg[i]));
+            // two scalar FMAs: packed, the operands' copies into pairs cost more than it saves
+            float2 C = make_float2(__fmaf_rn(ar, fp[i], seg[i]), __fmaf_rn(ab, fp[i], -seg[i]));
             const float2 Dj = Dq[dip_index(i)];
             C = __ffma2_rn(Dj, dip_neg(i) ? pS : mS, C);
             const H h = from2x(__ffma2_rn(mrho, diag(i) ? wd : wa, C));
@@ -309,8 +311,8 @@ __device__ __forceinline__ float node_viscosity(float rr, float rb, float inv_rh
 // - Instructions per node fell from 836 to 600 (FP16: 1140 to 800).
 // Measured at 8192^2 (drops, FP32): 1982 us per step before (33.9 GLUPS,
 // 4.9 TB/s), 1643 us now (40.9 GLUPS, 5.9 TB/s, 87 % of the measured copy);
-// 2048^2 143 -> 120 us; FP16 8192^2 2488 -> 1915 us, BF16 2614 -> 2030 us (bound
-// by issue: 66 % of the slots).  Two and four slots: 1851 and 1678 us.  Three
+// 2048^2 143 -> 120 us; FP16 8192^2 2488 -> 1893 us, BF16 2614 -> 2001 us (bound
+// by issue: 72 % of the slots).  Two and four slots: 1851 and 1678 us.  Three
 // CTAs per SM (168 registers): 1698 us.  256-column windows (two CTAs of eight
 // warps) 1930 us: fewer barrier domains to overlap.  The loop is unrolled
 // twice: four times saves the moves of the register FIFO (13 per row) but the
@@ -424,7 +426,8 @@ struct MarchF32 {
 
 // 16-bit storage (the record of Layout16): rows of records are copied as they
 // lie, and each is decoded once, by the thread of its own column, into FP32
-// populations in shared memory, from where stage A gathers as in FP32.
+// populations in shared memory (a (red, blue) pair per column and link), from
+// where stage A gathers as in FP32.
 // Decoding inside the gather, as the warp-specialised form did, decodes every
 // record twice (stages A and D) and each of its links with its neighbour's
 // reference.  A decoded plane keeps the rows its gather still needs: four of
@@ -439,8 +442,7 @@ struct March16 {
     static constexpr int kRefBytes = W * 8;           // (rho_R, rho_B), then (R_0, B_0), float2 per column
     static constexpr int kPairOff = 2 * kRefBytes;
     static constexpr int kSlotBytes = kPairOff + 12 * W * 4;
-    static constexpr int kDecRows = 24;                  // decoded rows per colour
-    static constexpr int kDecBytes = 2 * kDecRows * W * 4;
+    static constexpr int kDecBytes = 24 * W * 8;         // decoded rows, a (red, blue) pair per column
     static constexpr int kBytes = kSlots * kSlotBytes + kDecBytes + kMarchRows * W * 4;
     static constexpr int kLead = 3;                      // iterations that only decode
     // first decoded row of link i
@@ -485,8 +487,8 @@ struct March16 {
     };
 
     // The record of column t in a slot into the decoded rows (dec: column t),
-    // the links with c_y = 1 at s4 floats from their first row, the others at s2.
-    __device__ __forceinline__ static void decode(const char* slot, int t, float* dec, int s4, int s2,
+    // the links with c_y = 1 at s4 pairs from their first row, the others at s2.
+    __device__ __forceinline__ static void decode(const char* slot, int t, float2* dec, int s4, int s2,
                                                   const StepParams& P) {
         const float2 rho = reinterpret_cast<const float2*>(slot)[t];
         const float2 rest = reinterpret_cast<const float2*>(slot + kRefBytes)[t];
@@ -497,11 +499,7 @@ struct March16 {
         float2 c[9];
         Record::decode(rho, rest, raw, P, c);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            float* to = dec + (dec_row(i) * W + (lcy(i) > 0 ? s4 : s2));
-            to[0] = c[i].x;
-            to[kDecRows * W] = c[i].y;
-        }
+        for (int i = 0; i < 9; ++i) dec[dec_row(i) * W + (lcy(i) > 0 ? s4 : s2)] = c[i];
     }
 };
 // 1 KB reserved per CTA, and up to 512 B static in the batched kernel
@@ -532,7 +530,7 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
     const int r_first = T.y0 - 3 - kLead;
     const unsigned pop_addr = static_cast<unsigned>(__cvta_generic_to_shared(smem));
     // this thread's column of the decoded rows (16-bit storage) and of the stage rings
-    float* dec = reinterpret_cast<float*>(smem + L::kSlots * L::kSlotBytes) + t;
+    float2* dec = reinterpret_cast<float2*>(smem + L::kSlots * L::kSlotBytes) + t;
     float* ring = reinterpret_cast<float*>(smem + L::kBytes) - kMarchRows * W + t;
     auto row_ok = [&](int r) { return !WALLS || !T.wall || (r >= 0 && r < T.ny); };
     auto at_low = [&](int r) { return WALLS && T.wall && r == 0; };
@@ -655,9 +653,9 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
                         const int own = L::dec_row(lopp(i)) * W + (lcy(i) < 0 ? c0 * W + half : s2 * W);
                         const int row = L::dec_row(i) * W + (lcy(i) > 0 ? (c1 & 1) * W + ((c1 & 2) ? 2 * W - half : half)
                                                                         : (lcy(i) < 0 ? s2 ^ 1 : s2) * W);
-                        const float* at = dec + (wall ? own : row) + d;
-                        fr[i] = at[0];
-                        fb[i] = at[L::kDecRows * W];
+                        const float2 v = dec[(wall ? own : row) + d];
+                        fr[i] = v.x;
+                        fb[i] = v.y;
                     } else {
                         const float* at = reinterpret_cast<const float*>(smem + k % L::kSlots * L::kSlotBytes) + t + d;
                         fr[i] = at[i * W];

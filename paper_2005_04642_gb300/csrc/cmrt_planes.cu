@@ -962,7 +962,7 @@ constexpr int rs_edge(bool vjp, bool split) { return (split ? 0 : 1) + (vjp ? 3 
 constexpr int kRsFields = 15;
 
 template <int H, bool W, bool VJP, bool SPLIT>
-__global__ void __launch_bounds__(kRsX * H, 2)
+__global__ void __launch_bounds__(kRsX * H, SPLIT && H == 16 ? 3 : 2)
     k_rev_small(const float* __restrict__ post, const float* __restrict__ lam, const StepParams P,
                 const float* __restrict__ F, const float* __restrict__ S, float* __restrict__ lam_out,
                 double* __restrict__ partials, bool first) {
@@ -1010,6 +1010,16 @@ __global__ void __launch_bounds__(kRsX * H, 2)
     RevCollide r;
     float gx = 0.0f, gy = 0.0f, K = 0.0f;
     r.acc[0] = r.acc[1] = r.acc[2] = 0.0f;
+    // R4's own inputs; with 16 window rows loaded only there, so that 40 registers
+    // let three CTAs stand on an SM (512^2: 59.9 us per step against 62.7 with two;
+    // at 12 rows, 128^2, 15.0 against 13.5)
+    constexpr bool kLate = SPLIT && H == 16;
+    auto load_r4 = [&]() {
+        if (!SPLIT) return;
+        r.rnb = __ldcg(S + kRNB * n + o);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) r.fbar[i] = __ldcg(S + static_cast<size_t>(kFB0 + i) * n + o);
+    };
     if constexpr (SPLIT) {
         if (in) {
             w[kDv * kN] = __ldcg(S + kDIVUB * n + o);
@@ -1033,11 +1043,7 @@ __global__ void __launch_bounds__(kRsX * H, 2)
             r.rrb = __ldcg(S + kRRB * n + o);
             r.rbb = __ldcg(S + kRBB * n + o);
         }
-        if (inner(3)) {
-            r.rnb = __ldcg(S + kRNB * n + o);
-#pragma unroll
-            for (int i = 0; i < 9; ++i) r.fbar[i] = __ldcg(S + static_cast<size_t>(kFB0 + i) * n + o);
-        }
+        if (!kLate && inner(3)) load_r4();
     } else {
         if (in) {
             ux = __ldcg(F + kUX * n + o);
@@ -1137,6 +1143,7 @@ __global__ void __launch_bounds__(kRsX * H, 2)
     __syncthreads();
     // ---- R4: reverse of the gradients, rho^N, Phi' and the moments (k_rev_moments)
     if (inner(kD + 3)) {
+        if (kLate) load_r4();
         float rnb = r.rnb;
         rnb += gradT(w + kGxb_ * kN, true, 1.0f) + gradT(w + kGyb_ * kN, false, 1.0f);
         const float phb = gradT(w + kPxb * kN, true, 1.0f) + gradT(w + kPyb * kN, false, 1.0f);
