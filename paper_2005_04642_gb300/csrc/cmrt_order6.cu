@@ -5,14 +5,17 @@
 //
 // One node per thread: a CTA takes a window of 32 x H nodes, 22 x (H - 10) of
 // them its own, gathers each node's populations into registers and runs
-//   moments, chi, Phi' | grad rho^N, n-hat (halo 2) | K, G, u (halo 1) | the rest,
+//   moments, chi, Phi' | grad rho^N (halo 2) | K, G, u (halo 1) | the rest,
 // with a barrier between, the fields that a stencil reads in shared memory.
 // What bounds it: the launch and one load latency on small lattices, else
 // latency at one CTA of 1024 threads per SM (the window's halo makes the moments
 // 2x, H = 32, to 4x their work; whole warps of halo rows skip the collision).
-// Per step, as four passes over planes in memory -> here: 64^2 9.2 -> 2.7 us,
-// 256^2 11.2 -> 5.2, 512^2 21.4 -> 18.3, 1024 x 512 38.2 -> 34.2, 2048^2 302 ->
-// 279; one launch instead of four, and no 28 planes of scratch per node.
+// Per step, as four passes over planes in memory -> here: 64^2 9.2 -> 2.8 us,
+// 256^2 11.2 -> 5.4, 512^2 21.4 -> 19.3, 1024 x 512 38.2 -> 36.4, 2048^2 302 ->
+// 296; one launch instead of four, and no 28 planes of scratch per node.  The same
+// bits as the passes: a node's K takes the n-hat of its neighbours from their
+// gradients (n-hat kept in shared memory instead: 1024 x 512 34.2 us, but the
+// contraction of K then differs, and with walls the small u_y by 2e-4).
 #include <atomic>
 
 #include "cmrt_device.cuh"
@@ -26,6 +29,12 @@ __device__ __forceinline__ int wrap(int v, int n) {
     if (v >= 0 && v < n) return v;
     const int r = v % n;
     return r < 0 ? r + n : r;
+}
+__device__ __forceinline__ void normal_of(float gx, float gy, float& nx, float& ny) {
+    const float mag2 = fmaf(gx, gx, gy * gy);
+    const float inv = (mag2 >= kNormalTau * kNormalTau) ? rsqrtf(mag2) : 0.0f;
+    nx = -gx * inv;
+    ny = -gy * inv;
 }
 // App. B coefficients a_N
 __host__ __device__ constexpr float coef(int N) { return N == 1 ? 4.5f : (N == 2 ? -0.9f : 0.1f); }
@@ -48,7 +57,7 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
     const bool own = inner(kEdge) && xw < nx && yw < ny;
     const bool low = W && y == 0, high = W && y == ny - 1;
     float* w = sm + kX + threadIdx.x;  // this node in a field of the window
-    constexpr int kChiR = 0, kChiB = 1, kPhi = 2, kNx = 3, kNy = 4, kUx = 5, kUy = 6;
+    constexpr int kChiR = 0, kChiB = 1, kPhi = 2, kGx = 3, kGy = 4, kUx = 5, kUy = 6;
     // window offset of the row y + dy, or of its mirror beyond a wall
     auto row = [&](int dy) {
         int t = y + dy;
@@ -121,17 +130,27 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
         grad6(w + (red_minor ? kChiR : kChiB) * kN, gx, gy);
         gx *= red_minor ? 2.0f : -2.0f;
         gy *= red_minor ? 2.0f : -2.0f;
-        const float mag2 = fmaf(gx, gx, gy * gy);
-        const float inv = (mag2 >= kNormalTau * kNormalTau) ? rsqrtf(mag2) : 0.0f;
-        w[kNx * kN] = -gx * inv;
-        w[kNy * kN] = -gy * inv;
+        w[kGx * kN] = gx;
+        w[kGy * kN] = gy;
     }
     __syncthreads();
     // ---- K, G, u
     const float rho = rr + rb;
     float Gx = 0.0f, Gy = 0.0f, ux = 0.0f, uy = 0.0f;
     if (inner(4)) {
-        const float K = P.curvature_mode == 0 ? d_x(w + kNx * kN, 1.0f) + d_y(w + kNy * kN, -1.0f) : P.fixed_K;
+        float K = P.fixed_K;
+        if (P.curvature_mode == 0) {
+            // K = div n-hat with n-hat of the neighbours (y odd beyond a wall)
+            float nxv[9], nyv[9];
+#pragma unroll
+            for (int i = 1; i < 9; ++i) {
+                const bool mir = W && ((lcy(i) > 0 && high) || (lcy(i) < 0 && low));
+                const int o = (lcy(i) > 0 ? up : (lcy(i) < 0 ? dn : 0)) + lcx(i);
+                normal_of(w[kGx * kN + o], w[kGy * kN + o], nxv[i], nyv[i]);
+                if (W && mir) nyv[i] = -nyv[i];
+            }
+            K = ddx(nxv[8], nxv[4], nxv[1], nxv[3], nxv[7], nxv[5]) + ddy(nyv[2], nyv[6], nyv[1], nyv[3], nyv[7], nyv[5]);
+        }
         const float hk = P.half_sigma * K;
         Gx = fmaf(hk, gx, fmaf(rho, P.gacc_x, P.gvol_x));
         Gy = fmaf(hk, gy, fmaf(rho, P.gacc_y, P.gvol_y));
