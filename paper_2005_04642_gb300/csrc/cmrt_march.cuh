@@ -456,6 +456,7 @@ struct March16 {
     struct Copy {
         const char* two;   // this thread's chunk or column of the densities or rest populations, row 0
         const char* pair;  // of its first pair plane
+        unsigned x;        // without VEC: its column
         __device__ __forceinline__ void init(const Tile& T) {
             const int t = threadIdx.x;
             if (VEC) {
@@ -464,9 +465,7 @@ struct March16 {
                 pair = T.src + T.nodes * 16 + static_cast<size_t>(t / (W / 4)) * T.nodes * 4 +
                        static_cast<size_t>(wrap(T.x0 - kHalo + t % (W / 4) * 4, T.nx)) * 4;
             } else {
-                const size_t x = wrap(T.x0 - kHalo + t, T.nx);
-                two = T.src + x * 8;
-                pair = T.src + T.nodes * 16 + x * 4;
+                x = wrap(T.x0 - kHalo + t, T.nx);
             }
         }
         __device__ __forceinline__ void issue(const Tile& T, unsigned slot, int r) const {
@@ -478,10 +477,12 @@ struct March16 {
 #pragma unroll
                 for (int m = 0; m < 3; ++m) cp_async16(slot + kPairOff + (t + m * W) * 16, pair + (o + 4 * m * nodes) * 4);
             } else {
-                cp_async8(slot + t * 8, two + o * 8);
-                cp_async8(slot + kRefBytes + t * 8, two + (o + nodes) * 8);
+                const char* row = T.src + o * 8;
+                cp_async8(slot + t * 8, row + x * 8u);
+                cp_async8(slot + kRefBytes + t * 8, row + nodes * 8 + x * 8u);
+                row = T.src + nodes * 16 + o * 4;
 #pragma unroll
-                for (int q = 0; q < 12; ++q) cp_async4(slot + kPairOff + (q * W + t) * 4, pair + (o + q * nodes) * 4);
+                for (int q = 0; q < 12; ++q) cp_async4(slot + kPairOff + (q * W + t) * 4, row + q * nodes * 4 + x * 4u);
             }
         }
     };
@@ -1049,13 +1050,13 @@ dim3 small_grid(const StepParams& P, int H) {
 
 // Whether a step runs as k_small.  FP32, per step with 16 window rows: 18.3,
 // 22.4, 29.7 and 40.4 us at 640^2, 720^2, 800^2 and 900^2, whatever the width;
-// the march 21.2, 24.3, 29.7 and 28.0 us with 16-byte copies and 23.1, 38, 38
-// and 33.6 us with 4-byte ones (nx not a multiple of 4).  16-bit: 16.7, 24.5
+// the march 21.2, 22.4, 25.9 and 27.3 us with 16-byte copies; at 801^2 and 901^2,
+// with 4-byte ones (nx not a multiple of 4), 29.6 and 33.2 us.  16-bit: 16.7, 24.5
 // and 29.9 us at 512^2, 640^2 and 720^2 against the march's 18.8, 24.4 and 30.7.
 template <class L>
 bool use_small(const StepParams& P) {
     const long nodes = static_cast<long>(P.nx) * P.ny;
-    const long limit = L::kDecode ? 450000 : 600000;
+    const long limit = L::kDecode ? 330000 : 600000;
     const int rows = 16 - 2 * small_halo<L>();
     return nodes <= ((P.nx % 4) == 0 ? limit : limit + 100000) && P.ny <= 65535 * rows;  // grid rows
 }
@@ -1113,11 +1114,16 @@ cudaError_t launch_march(const void* src, void* dst, const StepParams& P, int ro
         if (use_small<L>(P)) return launch_small_any<L, MODE>(src, dst, P, fo, flag, s);
     }
     const bool vec = (P.nx % 4) == 0;
-    const bool walls = P.wall_y != 0;
+    // 16-bit rows copied 4 bytes at a time take the form for walls, which is right for
+    // any lattice: the periodic one spills 12 bytes, and its copies through L1 evict
+    // them (BF16 3883 x 634 180 us per step against 116)
+    const bool walls = P.wall_y != 0 || (L::kDecode && !vec);
     if (vec && walls) return launch_march_one<L, true, true, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
     if (vec) return launch_march_one<L, true, false, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
-    if (walls) return launch_march_one<L, false, true, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
-    return launch_march_one<L, false, false, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
+    if constexpr (!L::kDecode) {
+        if (!walls) return launch_march_one<L, false, false, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
+    }
+    return launch_march_one<L, false, true, MODE, PRE>(src, dst, P, rows, fo, flag, partials, s);
 }
 
 }  // namespace
