@@ -52,30 +52,30 @@ dim3 chain_grid(int nx, int ny, int rows) {
 
 int chain_rows(int nx, int ny, int sms, int precision) {
     // Rows per CTA.  A CTA spends rows + 7 row iterations (7 fill the
-    // pipeline); an iteration takes longer the more CTAs share its SM (FP32,
-    // 1024 columns and up: 0.75 us alone on an SM, 1.45 us with four, hence
-    // 0.55 + 0.23 n).  Within one wave the fullest SM sets the time, by a
-    // quarter more where the state is beyond L2 (2048^2: 122 us with 64 rows in
-    // one wave, 129 with 32; 4096^2: 505 us with 241 rows, 439 with 64).  Past one
-    // wave the hardware hands out CTAs as others finish, which evens out the
-    // SMs' different speeds (two dies), and half a CTA's time is lost at the
-    // end.  Measured at 8192^2: 36.3, 38.0, 40.4, 40.6, 40.9, 40.5 and 39.5
-    // GLUPS with 512, 256, 192, 128, 96, 64 and 48 rows; at 4096^2 26.8, 32.8,
-    // 36.1, 37.8, 38.2, 38.2 and 37.3 with 512, 256, 128, 96, 64, 48 and 32.
-    // The 16-bit storage keeps whole waves of two CTAs per SM and 8 fill rows.
+    // pipeline, 9 with 16-bit storage); an iteration takes longer the more CTAs
+    // share its SM: 0.79, 0.95, 1.40 and 1.47 us with one to four (FP32, states
+    // within L2).  Within one wave the fullest SM sets the time, by a quarter
+    // more where the state is beyond L2 (2048^2: 120 us with 64 rows in one wave,
+    // 129 with 32; 4096^2: 505 us with 241 rows, 435 with 64).  Past one wave the
+    // hardware hands out CTAs as others finish, which evens out the SMs'
+    // different speeds (two dies), and half a CTA's time is lost at the end.
+    // Measured at 8192^2: 36.3, 38.0, 40.4, 40.6, 40.9, 40.5 and 39.5 GLUPS with
+    // 512, 256, 192, 128, 96, 64 and 48 rows; at 4096^2 26.8, 32.8, 36.1, 37.8,
+    // 38.2, 38.2 and 37.3 with 512, 256, 128, 96, 64, 48 and 32.
+    constexpr double kUs[4] = {0.79, 0.95, 1.40, 1.47};
+    static_assert(march_ctas<kWin>() == 4, "a time per CTA count");
     const int strips = (nx + kTileX - 1) / kTileX;
     const int n_sms = sms > 0 ? sms : 1;
     const int fill = precision == kPrecF32 ? 7 : 9;
-    const double slots = static_cast<double>(march_ctas<kWin>()) * n_sms;
+    const double slots = 4.0 * n_sms;
     const bool beyond_l2 = 144.0 * nx * ny > 126e6;
     int best = 8;
     double best_cost = -1.0;
     for (int rows = 1; rows <= 512; rows += rows < 32 ? 1 : 8) {
         const long ctas = static_cast<long>(strips) * ((ny + rows - 1) / rows);
         const double waves = ctas / slots;
-        double cost;
-        if (waves <= 1.0) cost = (rows + fill) * (0.55 + 0.23 * ((ctas + n_sms - 1) / n_sms)) * (beyond_l2 ? 1.25 : 1.0);
-        else cost = (rows + fill) * (0.55 + 0.23 * march_ctas<kWin>()) * (waves + 0.5);
+        const double cost = (rows + fill) * (waves <= 1.0 ? kUs[(ctas - 1) / n_sms] * (beyond_l2 ? 1.25 : 1.0)
+                                                          : kUs[3] * (waves + 0.5));
         if (best_cost < 0.0 || cost < best_cost) {
             best_cost = cost;
             best = rows;
