@@ -86,6 +86,29 @@ constexpr float kNormalTau = 1e-9f;
 
 __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
 
+// A running sum of a few FP32 terms as an FP32 pair: every addition's rounding
+// error, computed exactly (Knuth's TwoSum), goes to lo, so that hi + lo carries
+// about 48 bits.  GB300's FP64 unit takes an SM 16 cycles per warp instruction,
+// and a conversion and an addition per term bound the diagnostics pass (2048^2:
+// 142 us; with pairs 87).  take() hands the sum to an FP64 accumulator (exactly)
+// and starts anew; after at most eight terms the pair's own error, below 2^-45
+// of the sum, stays at the level of the FP64 accumulation.
+struct Sum2 {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = __fadd_rn(hi, x);
+        const float b = __fsub_rn(s, hi);
+        const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
+        hi = s;
+        lo = __fadd_rn(lo, e);
+    }
+    __device__ __forceinline__ double take() {
+        const double v = static_cast<double>(hi) + static_cast<double>(lo);
+        hi = lo = 0.0f;
+        return v;
+    }
+};
+
 // Segregation term of link i, w_i (s . c-hat_i) for a vector s (Eq. eq_re_color
 // with phi_i = w_i phim folded into s).
 __device__ __forceinline__ void segregation(float sx, float sy, float (&seg)[9]) {

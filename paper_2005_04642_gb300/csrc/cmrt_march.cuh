@@ -543,8 +543,9 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
         const int j = k - kLead - 3 - d;
         return MODE == Pass::StepFields && own_col && j >= 0 && j < rows;
     };
+    // (a plane's row address is common to the CTA)
     auto fwd = [&](int plane, int r) -> float& {
-        return fo.fwd[static_cast<size_t>(plane) * T.nodes + static_cast<size_t>(r) * T.nx + gx_own];
+        return (fo.fwd + static_cast<size_t>(plane) * T.nodes + static_cast<size_t>(r) * T.nx)[static_cast<unsigned>(gx_own)];
     };
     // ring rows (column t): field f of the row in slot c; slots 0, 1 and 2, 3 of an
     // iteration trade places every two iterations
@@ -571,6 +572,9 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
 #pragma unroll
     for (int j = 0; j < L::kSlots - 1; ++j) issue(j);
 
+    // diagnostics: up to eight rows' sums, and the fastest node so far
+    Sum2 sum_r, sum_b, sum_jx, sum_jy, best;
+    float best_ux = 0.0f, best_uy = 0.0f;
     // what the later stages of this column need.  f, rho_R, rho_B and j: before an
     // even iteration slots 0 .. 3 hold rows r - 1 .. r - 4, before an odd one
     // slots 1, 0, 3, 2; grad rho^N and G alternate
@@ -620,11 +624,23 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
                 const float mx = (F[1] + F[7] + F[8]) - (F[3] + F[4] + F[5]);
                 const float my = (F[1] + F[2] + F[3]) - (F[5] + F[6] + F[7]);
                 if (isfinite(rho)) {
-                    acc.r += drr;
-                    acc.b += drb;
-                    acc.jx += mx;
-                    acc.jy += my;
-                    acc.u2 = fmax(acc.u2, static_cast<double>(ux) * ux + static_cast<double>(uy) * uy);
+                    sum_r.add(drr);
+                    sum_b.add(drb);
+                    sum_jx.add(mx);
+                    sum_jy.add(my);
+                    // |u|^2 as an FP32 pair, to find the node whose FP64 value is the largest
+                    const float p = __fmul_rn(ux, ux), q = __fmul_rn(uy, uy);
+                    Sum2 u2;
+                    u2.add(p);
+                    u2.add(q);
+                    const float lo = u2.lo + (__fmaf_rn(ux, ux, -p) + __fmaf_rn(uy, uy, -q));
+                    const float top = __fadd_rn(u2.hi, lo), rest = lo - (top - u2.hi);
+                    if (top > best.hi || (top == best.hi && rest > best.lo)) {
+                        best.hi = top;
+                        best.lo = rest;
+                        best_ux = ux;
+                        best_uy = uy;
+                    }
                 } else {
                     acc.bad += 1.0;
                 }
@@ -780,7 +796,15 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
         iteration(Const<0>{}, k);
         if (k + 1 < iters) iteration(Const<1>{}, k + 1);
         half = 2 * W - half;
+        if (MODE == Pass::Diag && ((k & 6) == 6 || k + 2 >= iters)) {
+            acc.r += sum_r.take();
+            acc.b += sum_b.take();
+            acc.jx += sum_jx.take();
+            acc.jy += sum_jy.take();
+        }
     }
+    if (MODE == Pass::Diag)
+        acc.u2 = fmax(acc.u2, static_cast<double>(best_ux) * best_ux + static_cast<double>(best_uy) * best_uy);
     cp_wait<0>();
 }
 
