@@ -90,7 +90,7 @@ __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
 // error, computed exactly (Knuth's TwoSum), goes to lo, so that hi + lo carries
 // about 48 bits.  GB300's FP64 unit takes an SM 16 cycles per warp instruction,
 // and a conversion and an addition per term bound the diagnostics pass (2048^2:
-// 142 us; with pairs 87).  take() hands the sum to an FP64 accumulator (exactly)
+// 142 us; with pairs 89).  take() hands the sum to an FP64 accumulator (exactly)
 // and starts anew; after at most eight terms the pair's own error, below 2^-45
 // of the sum, stays at the level of the FP64 accumulation.
 struct Sum2 {

@@ -428,7 +428,7 @@ struct MarchF32 {
 // lie, and each is decoded once, by the thread of its own column, into FP32
 // populations in shared memory (a (red, blue) pair per column and link), from
 // where stage A gathers as in FP32.
-// Decoding inside the gather, as the warp-specialised form did, decodes every
+// Decoding inside the gather, as the earlier two-group form did, decodes every
 // record twice (stages A and D) and each of its links with its neighbour's
 // reference.  A decoded plane keeps the rows its gather still needs: four of
 // the links with c_y = 1 (rows r - 1 .. r + 2 of iteration r; four for a
@@ -624,10 +624,18 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
                 const float mx = (F[1] + F[7] + F[8]) - (F[3] + F[4] + F[5]);
                 const float my = (F[1] + F[2] + F[3]) - (F[5] + F[6] + F[7]);
                 if (isfinite(rho)) {
-                    sum_r.add(drr);
-                    sum_b.add(drb);
-                    sum_jx.add(mx);
-                    sum_jy.add(my);
+                    // (values whose FP32 sums or squares could overflow or underflow go to FP64)
+                    if (fmaxf(fmaxf(fabsf(drr), fabsf(drb)), fmaxf(fabsf(mx), fabsf(my))) < 1e30f) {
+                        sum_r.add(drr);
+                        sum_b.add(drb);
+                        sum_jx.add(mx);
+                        sum_jy.add(my);
+                    } else {
+                        acc.r += drr;
+                        acc.b += drb;
+                        acc.jx += mx;
+                        acc.jy += my;
+                    }
                     // |u|^2 as an FP32 pair, to find the node whose FP64 value is the largest
                     const float p = __fmul_rn(ux, ux), q = __fmul_rn(uy, uy);
                     Sum2 u2;
@@ -635,7 +643,10 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
                     u2.add(q);
                     const float lo = u2.lo + (__fmaf_rn(ux, ux, -p) + __fmaf_rn(uy, uy, -q));
                     const float top = __fadd_rn(u2.hi, lo), rest = lo - (top - u2.hi);
-                    if (top > best.hi || (top == best.hi && rest > best.lo)) {
+                    if (!(top > 1e-28f && top < 1e30f)) {
+                        if (ux != 0.0f || uy != 0.0f)
+                            acc.u2 = fmax(acc.u2, static_cast<double>(ux) * ux + static_cast<double>(uy) * uy);
+                    } else if (top > best.hi || (top == best.hi && rest > best.lo)) {
                         best.hi = top;
                         best.lo = rest;
                         best_ux = ux;

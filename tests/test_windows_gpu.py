@@ -102,3 +102,34 @@ def test_reverse_step_by_windows_matches_plane_passes(nx, ny, wall):
         assert all(abs(x - y) <= 1e-5 * abs(y) + 1e-7 * top for x, y in zip(a, b)), (a, b)
     assert (r0 - r2).abs().max() <= 1e-5 * r2.abs().max()
     assert (v0 - v2).abs().max() <= 1e-5 * v2.abs().max()
+
+
+@pytest.mark.parametrize("precision", [1, 2], ids=["bf16", "fp16"])
+def test_march_with_4_byte_copies_gives_the_bits_of_16_byte_ones(precision):
+    """An odd width beyond the windows' range, a flow that is uniform along x: each
+    column equals any column of a lattice whose width is a multiple of 4."""
+    cols = []
+    for nx in (757, 760):
+        d = I.base_params(nx, 600, wall_y=False, g_acc=(1e-5, -2e-5), precision=precision)
+        rn = np.repeat(np.tanh(np.sin(2 * np.pi * np.arange(600) / 600) * 20)[:, None], nx, 1).astype(np.float32)
+        lat = cm.Lattice(d, rn, None)
+        lat.step(3)
+        p = lat.populations()
+        assert torch.equal(p, p[..., :1].expand_as(p))
+        cols.append(p[..., 0])
+        lat.close()
+    assert torch.equal(*cols)
+
+
+@pytest.mark.parametrize("g", [1e-24, 1e-14, 1e-3, 1e19], ids=str)
+@pytest.mark.parametrize("precision", [0, 2], ids=["fp32", "fp16"])
+def test_diagnosed_speed_over_the_range_of_fp32(g, precision):
+    """max|u| where |u|^2 is below, within and above FP32's range, against the
+    fields' u: the two forms may round u by a few FP32 spacings differently."""
+    d = I.base_params(40, 24, wall_y=False, g_acc=(g, -2.0 * g), precision=precision)
+    lat = cm.Lattice(d, np.ones((24, 40), np.float32), None)
+    f = lat.fields()
+    want = float(torch.hypot(f["ux"].double(), f["uy"].double()).max())
+    assert want >= g
+    assert lat.diagnostics()["umax"] == pytest.approx(want, rel=1e-6, abs=0.0)
+    lat.close()
