@@ -443,7 +443,7 @@ def run_cmrt(args, rank, world, local_rank):
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "peak_source": peak_kind, "nominal_peak": NOMINAL_HBM_GBS, "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
                 "traffic": recorded_traffic(cells),
-                "algorithmic_bytes_per_launch": BYTES_PER_CELL * cells, "kernel": "k_chain<Step>",
+                "algorithmic_bytes_per_launch": BYTES_PER_CELL * cells, "kernel": "k_march<Step>",
                 "source_sha": kernel_source_sha()}
     cpu = None
     if world == 1 and not args.no_cpu_baseline:
