@@ -536,6 +536,7 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
     auto row_ok = [&](int r) { return !WALLS || !T.wall || (r >= 0 && r < T.ny); };
     auto at_low = [&](int r) { return WALLS && T.wall && r == 0; };
     auto at_high = [&](int r) { return WALLS && T.wall && r == T.ny - 1; };
+    __shared__ float density[MODE == Pass::Fields ? 2 * W : 1];  // fields: rho_R, rho_B of D's row
     const int gx_own = T.x0 + t - kHalo;
     const bool own_col = t >= kHalo && t < W - kHalo && gx_own < T.nx;
     // iteration k handles own row k - kLead - 3 - d at a stage d rows behind stage A
@@ -586,11 +587,28 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
         constexpr int c1 = (c0 + 3) & 3, c2 = (c0 + 2) & 3, c3 = (c0 + 1) & 3;  // of rows r - 1, r - 2, r - 3
         const int r = r_first + k;
         if (!L::kDecode) cp_wait<L::kSlots - 2>();
+        if constexpr (MODE == Pass::Fields) {  // read by D; its last readers are two barriers back
+            density[t] = rr[old];
+            density[W + t] = rb[old];
+        }
         __syncthreads();
         issue(k + L::kSlots - 1);  // into the slot read in the last iteration
         // ---- D: row r - 4 (FIFO slot c0): rows r - 3, r - 4, r - 5 of the rings in slots c3, c0, c1
         const int yd = r - 4;
-        if (k >= 7 + kLead && own_col) {
+        if constexpr (MODE == Pass::Fields) {
+            // thread t writes own column t (window column t + 4): warps then start on
+            // 32-byte sectors, which host memory wants (page-locked outputs, 8192^2: 8.02
+            // ms, 8.95 where each thread wrote its own column; device outputs the same)
+            if (k >= 7 + kLead && t < W - 2 * kHalo && T.x0 + t < T.nx) {
+                const size_t o = static_cast<size_t>(yd) * T.nx + (T.x0 + t);
+                const float drr = density[t + kHalo], drb = density[W + t + kHalo];
+                if (fo.rho_r) fo.rho_r[o] = drr;
+                if (fo.rho_b) fo.rho_b[o] = drb;
+                if (fo.ux) fo.ux[o] = R(kUx, c0)[kHalo];
+                if (fo.uy) fo.uy[o] = R(kUy, c0)[kHalo];
+                if (fo.p) fo.p[o] = fmaf(P.cs2_r, drr, P.cs2_b * drb);
+            }
+        } else if (k >= 7 + kLead && own_col) {
             const float drr = rr[old], drb = rb[old];
             const float rho = drr + drb;
             const float ux = R(kUx, c0)[0], uy = R(kUy, c0)[0];
@@ -612,13 +630,6 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
                 else
                     store_recoloured_f32(reinterpret_cast<float*>(T.dst) + static_cast<size_t>(yd) * T.nx, gx_own, T.nodes,
                                          fp, drr, drb, inv_rho, sg * ex, sg * ey);
-            } else if (MODE == Pass::Fields) {
-                const size_t o = static_cast<size_t>(yd) * T.nx + gx_own;
-                if (fo.rho_r) fo.rho_r[o] = drr;
-                if (fo.rho_b) fo.rho_b[o] = drb;
-                if (fo.ux) fo.ux[o] = ux;
-                if (fo.uy) fo.uy[o] = uy;
-                if (fo.p) fo.p[o] = fmaf(P.cs2_r, drr, P.cs2_b * drb);
             } else {
                 const float* F = f[old];
                 const float mx = (F[1] + F[7] + F[8]) - (F[3] + F[4] + F[5]);
