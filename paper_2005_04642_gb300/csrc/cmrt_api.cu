@@ -1784,7 +1784,7 @@ extern "C" cmrt_status cmrt_step_vjp(cmrt_ctx* h, const float* lam_next, float* 
 // reverse steps len - 2 .. 0 skip that recomputation.  Recorded on the first
 // use of (len, a) -- on a private stream, so the caller's stream may be any
 // -- and replayed afterwards; *launches receives its kernel count.  sp: the
-// call's parameters (fused reverse kernels where it uses forward fields).
+// call's parameters (kAdjWritten where it uses forward fields).
 cmrt_status adj_segment_graph(Ctx* c, const cmrt::StepParams& sp, int64_t len, int a, cudaGraphExec_t* out,
                               int64_t* launches) {
     const bool emit = c->adj_fields && cmrt::adj_fused(sp) && len > 1 &&
@@ -1867,13 +1867,13 @@ extern "C" cmrt_status cmrt_adjoint(cmrt_ctx* h, int64_t nsteps, int32_t ckpt_ev
     // forward, keeping P_{kK-1} (relative to the current time) as checkpoint k
     CK(c, cudaMemcpyAsync(c->adj_ckpt, c->buf[c->cur], state, cudaMemcpyDeviceToDevice, c->stream));
     // Forward fields from the forward steps where the field buffer could be
-    // had: then every reverse step of the call runs fused (the same kernels
-    // whichever source a state's fields come from, so the checkpoint interval
-    // does not change the result); otherwise the lattice-size rule decides.
+    // had: then every reverse step of the call runs as kernels that can read them
+    // (the same ones whichever source a state's fields come from, so the checkpoint
+    // interval does not change the result); otherwise the lattice-size rule decides.
     const size_t need = K == 1 ? static_cast<size_t>(nsteps) : seg - 1;
     const bool use_fields = cmrt::adj_fields_usable(c->sp) && need > 0 && c->adj_fields && c->adj_fields_cap >= need;
     cmrt::StepParams spa = c->sp;
-    if (use_fields) spa.adjoint_fused = 1;
+    if (use_fields && spa.adjoint_fused == 0) spa.adjoint_fused = cmrt::kAdjWritten;
     // every state kept: each forward step writes the fields of the state it reads
     const bool emit_all = K == 1 && use_fields;
     const size_t nf = static_cast<size_t>(cmrt::kFwdPlanes) * n;

@@ -34,13 +34,17 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     }(static_cast<Args&&>(args)...);
 }
 
-// Parameters of one step in the form the kernels use: FP32 coefficients
-// derived once on the host (in FP64) from cmrt_params.
 // Population storage in HBM (cmrt_params.precision).
 constexpr int kPrecF32 = 0;
 constexpr int kPrecB16 = 1;
 constexpr int kPrecF16 = 2;
 
+// Reverse kernels of a call left to the automatic choice whose forward steps write
+// the forward fields: windows or row wavefronts, which can read them.
+constexpr int kAdjWritten = 3;
+
+// Parameters of one step in the form the kernels use: FP32 coefficients
+// derived once on the host (in FP64) from cmrt_params.
 struct StepParams {
     int nx, ny, wall_y;
     int precision;                 // kPrecF32 / kPrecB16 / kPrecF16
@@ -50,7 +54,7 @@ struct StepParams {
     float dev_scale, dev_unscale;  // 16-bit deviations are stored as d * dev_scale (a power of two)
     int visc_mode, curvature_mode, ghost_N_mode;
     int stencil_order;             // 2: compact gradients; 6: App. B for grad rho^N and grad Phi'
-    int adjoint_fused;              // 0: automatic, 1: fused reverse tail, 2: plane passes
+    int adjoint_fused;              // cmrt_params.adjoint_fused, or kAdjWritten
     float inv_rho0_r, inv_rho0_b;  // colour index (Eq. equ_rhoN_def)
     float alpha_r, alpha_b;        // rest weights phi_0 (Eq. eq_phi)
     float kphi_r, kphi_b;          // 9/5 (1 - alpha_C): phi_i = w_i (kphi_r rho_R + kphi_b rho_B) / rho
@@ -194,11 +198,12 @@ int adj_launches_per_step(const StepParams& P, bool vjp = false);
 // recompute them (used only where adj_fused(P)).
 cudaError_t launch_adjoint_step(const float* post, const float* lam_post, const StepParams& P, float* scratch,
                                 double* partials, float* lam_prev, cudaStream_t s, const float* fwd = nullptr);
-// whether one reverse step runs as the fused kernels (compact stencil, lattice large enough or asked for)
+// whether one reverse step can read written forward fields: it runs by windows or
+// as row wavefronts (compact stencil; by the lattice's size, or asked for)
 bool adj_fused(const StepParams& P);
-// whether the fused kernels may read forward fields written by the forward
-// steps (compact stencil, plane passes not asked for); a call that uses such
-// fields runs all its reverse steps fused
+// whether a call's forward steps may write forward fields (compact stencil, plane
+// passes not asked for); with adjoint_fused 0 all its reverse steps then run as
+// kAdjWritten says
 bool adj_fields_usable(const StepParams& P);
 // cmrt_step_vjp by windows (small lattices): lam_next is dJ/df(t+1) and lam
 // receives dJ/df(t), both in the public layout.  The rows of partials used:

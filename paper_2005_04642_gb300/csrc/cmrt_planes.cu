@@ -1240,11 +1240,13 @@ int tail_rows(int nx, int ny) {
     return rows;
 }
 
-// fused kernels or plane passes (compact stencil): as asked, else the fused
-// kernels where the lattice fills 16-row segments in two waves -- on smaller
-// lattices their fill rows per segment cost more than the launches they save
+// row wavefronts or plane passes (compact stencil, where rev_small does not hold):
+// as asked, wavefronts for written fields, else wavefronts where the lattice fills
+// 16-row segments in two waves -- on smaller lattices their fill rows per segment
+// cost more than the launches they save
 bool use_fused(const StepParams& P) {
-    return P.adjoint_fused == 1 || (P.adjoint_fused == 0 && tail_rows(P.nx, P.ny) >= 16);
+    return P.adjoint_fused == 1 || P.adjoint_fused == kAdjWritten ||
+           (P.adjoint_fused == 0 && tail_rows(P.nx, P.ny) >= 16);
 }
 
 template <bool W, bool EXPAND>
@@ -1583,8 +1585,8 @@ void forward_planes(const float* post, const StepParams& P, float* S, cudaStream
     k_fwd_force<W><<<g, kAT, 0, s>>>(P, S);
 }
 
-// The reverse step by windows: compact stencil, not with the plane passes asked
-// for, up to 400 000 nodes in an adjoint sweep, up to 900 000 in a step VJP
+// The reverse step by windows: compact stencil, neither the row wavefronts nor the
+// plane passes asked for, up to 400 000 nodes in an adjoint sweep, up to 900 000 in a step VJP
 // (whose alternative is the plane passes or recomputes the forward fields in a
 // row wavefront); the whole form up to 9000.  Measured, us per step of an
 // adjoint call with checkpoints (its forward run and replay included), before
@@ -1596,7 +1598,8 @@ void forward_planes(const float* post, const StepParams& P, float* S, cudaStream
 constexpr long kRevSweepNodes = 400000, kRevVjpNodes = 900000, kRevWholeNodes = 9000;
 long lattice_nodes(const StepParams& P) { return static_cast<long>(P.nx) * P.ny; }
 bool rev_small(const StepParams& P, bool vjp) {
-    return P.stencil_order == 2 && P.adjoint_fused != 2 && lattice_nodes(P) <= (vjp ? kRevVjpNodes : kRevSweepNodes);
+    return P.stencil_order == 2 && (P.adjoint_fused == 0 || P.adjoint_fused == kAdjWritten) &&
+           lattice_nodes(P) <= (vjp ? kRevVjpNodes : kRevSweepNodes);
 }
 bool rev_whole(const StepParams& P) { return lattice_nodes(P) <= kRevWholeNodes; }
 dim3 rev_small_grid(const StepParams& P, int H, bool vjp, bool split) {
