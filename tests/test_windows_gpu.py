@@ -133,3 +133,20 @@ def test_diagnosed_speed_over_the_range_of_fp32(g, precision):
     assert want >= g
     assert lat.diagnostics()["umax"] == pytest.approx(want, rel=1e-6, abs=0.0)
     lat.close()
+
+
+# all widths copy 16 bytes at a time: strips of 88 own columns (96-column windows) and of 120
+@pytest.mark.parametrize("precision", [0, 1, 2], ids=["fp32", "bf16", "fp16"])
+@pytest.mark.parametrize("walls", [(False, False), (True, True), (False, True)], ids=["periodic", "walls", "mixed"])
+@pytest.mark.parametrize("shapes", [[(88, 40), (176, 23), (256, 70), (84, 9)], [(120, 64), (240, 31), (112, 5)]],
+                         ids=["window96", "window128"])
+def test_batches_with_16_byte_copies_give_the_bits_of_windows(shapes, walls, precision):
+    members = [_setup(nx, ny, walls[k % 2], precision=precision) for k, (nx, ny) in enumerate(shapes)]
+    b = cm.Batch(members)
+    b.step(3)
+    for k, m in enumerate(members):
+        lat = cm.Lattice(*m)
+        lat.step(3)
+        assert torch.equal(b.member(k).populations(), lat.populations()), (m[0]["nx"], m[0]["ny"])
+        lat.close()
+    b.close()
