@@ -86,26 +86,45 @@ constexpr float kNormalTau = 1e-9f;
 
 __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
 
-// A running sum of a few FP32 terms as an FP32 pair: every addition's rounding
-// error, computed exactly (Knuth's TwoSum), goes to lo, so that hi + lo carries
-// about 48 bits.  GB300's FP64 unit takes an SM 16 cycles per warp instruction,
-// and a conversion and an addition per term bound the diagnostics pass (2048^2:
-// 142 us; with pairs 89).  take() hands the sum to an FP64 accumulator (exactly)
-// and starts anew; after at most eight terms the pair's own error, below 2^-45
-// of the sum, stays at the level of the FP64 accumulation.
-struct Sum2 {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = __fadd_rn(hi, x);
-        const float b = __fsub_rn(s, hi);
-        const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
-        hi = s;
-        lo = __fadd_rn(lo, e);
+// a + b as its FP32 rounding (returned) and the exact rest e (Knuth's TwoSum).
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+    const float s = __fadd_rn(a, b);
+    const float c = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, c)), __fsub_rn(b, c));
+    return s;
+}
+
+// The same for a pair of sums, as packed FP32x2 operations (a - b as b * -1 + a: one rounding).
+__device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& e) {
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    auto minus = [&](float2 x, float2 y) { return __ffma2_rn(y, m1, x); };
+    const float2 s = __fadd2_rn(a, b);
+    const float2 c = minus(s, a);
+    e = __fadd2_rn(minus(a, minus(s, c)), minus(b, c));
+    return s;
+}
+
+// A running pair of sums of up to eight FP32 terms in three FP32 parts: hi takes the
+// terms, mid the exact rests of its additions, lo the exact rests of mid's.  Only lo's
+// own additions round: with S the sum of the terms' magnitudes, mid stays below
+// 2^-21 S, lo below 2^-42 S and its error below 2^-63 S, so that the sums that take()
+// adds to FP64 accumulators are rounded there alone, less often than by an FP64
+// addition per term.  GB300's FP64 unit takes an SM 16 cycles per warp
+// instruction: a conversion and an addition per term bounded the diagnostics pass
+// (a call on 2048^2 154 us, on 8192 x 4096 1038; with Sum3 115 and 661; with hi
+// and lo alone, whose rest rounds at 2^-46 of the terms, 109 and 619).
+struct Sum3 {
+    float2 hi = {0.0f, 0.0f}, mid = {0.0f, 0.0f}, lo = {0.0f, 0.0f};
+    __device__ __forceinline__ void add(float x, float y) {
+        float2 e, e2;
+        hi = two_sum(hi, make_float2(x, y), e);
+        mid = two_sum(mid, e, e2);
+        lo = __fadd2_rn(lo, e2);
     }
-    __device__ __forceinline__ double take() {
-        const double v = static_cast<double>(hi) + static_cast<double>(lo);
-        hi = lo = 0.0f;
-        return v;
+    __device__ __forceinline__ void take(double& x, double& y) {
+        x += static_cast<double>(hi.x) + (static_cast<double>(mid.x) + static_cast<double>(lo.x));
+        y += static_cast<double>(hi.y) + (static_cast<double>(mid.y) + static_cast<double>(lo.y));
+        hi = mid = lo = make_float2(0.0f, 0.0f);
     }
 };
 

@@ -574,8 +574,8 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
     for (int j = 0; j < L::kSlots - 1; ++j) issue(j);
 
     // diagnostics: up to eight rows' sums, and the fastest node so far
-    Sum2 sum_r, sum_b, sum_jx, sum_jy, best;
-    float best_ux = 0.0f, best_uy = 0.0f;
+    Sum3 sum_mass, sum_mom;
+    float best_hi = 0.0f, best_lo = 0.0f, best_ux = 0.0f, best_uy = 0.0f;
     // what the later stages of this column need.  f, rho_R, rho_B and j: before an
     // even iteration slots 0 .. 3 hold rows r - 1 .. r - 4, before an odd one
     // slots 1, 0, 3, 2; grad rho^N and G alternate
@@ -637,31 +637,30 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
                 if (isfinite(rho)) {
                     // (values whose FP32 sums or squares could overflow or underflow go to FP64)
                     if (fmaxf(fmaxf(fabsf(drr), fabsf(drb)), fmaxf(fabsf(mx), fabsf(my))) < 1e30f) {
-                        sum_r.add(drr);
-                        sum_b.add(drb);
-                        sum_jx.add(mx);
-                        sum_jy.add(my);
+                        sum_mass.add(drr, drb);
+                        sum_mom.add(mx, my);
                     } else {
                         acc.r += drr;
                         acc.b += drb;
                         acc.jx += mx;
                         acc.jy += my;
                     }
-                    // |u|^2 as an FP32 pair, to find the node whose FP64 value is the largest
+                    // |u|^2 as an FP32 pair, good to 2^-46, finds the fastest node, whose FP64
+                    // value counts; of nodes closer than the pairs can tell (2^-42) each does
                     const float p = __fmul_rn(ux, ux), q = __fmul_rn(uy, uy);
-                    Sum2 u2;
-                    u2.add(p);
-                    u2.add(q);
-                    const float lo = u2.lo + (__fmaf_rn(ux, ux, -p) + __fmaf_rn(uy, uy, -q));
-                    const float top = __fadd_rn(u2.hi, lo), rest = lo - (top - u2.hi);
-                    if (!(top > 1e-28f && top < 1e30f)) {
-                        if (ux != 0.0f || uy != 0.0f)
-                            acc.u2 = fmax(acc.u2, static_cast<double>(ux) * ux + static_cast<double>(uy) * uy);
-                    } else if (top > best.hi || (top == best.hi && rest > best.lo)) {
-                        best.hi = top;
-                        best.lo = rest;
+                    float e;
+                    const float s = two_sum(p, q, e);
+                    const float lo = e + (__fmaf_rn(ux, ux, -p) + __fmaf_rn(uy, uy, -q));
+                    const float top = __fadd_rn(s, lo), rest = lo - (top - s);
+                    const bool usual = top > 1e-28f && top < 1e30f;
+                    const float lead = (top - best_hi) + (rest - best_lo), near = 0x1p-42f * top;
+                    if (usual && lead > near) {
+                        best_hi = top;
+                        best_lo = rest;
                         best_ux = ux;
                         best_uy = uy;
+                    } else if (usual ? lead >= -near && (ux != best_ux || uy != best_uy) : ux != 0.0f || uy != 0.0f) {
+                        acc.u2 = fmax(acc.u2, static_cast<double>(ux) * ux + static_cast<double>(uy) * uy);
                     }
                 } else {
                     acc.bad += 1.0;
@@ -819,10 +818,8 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
         if (k + 1 < iters) iteration(Const<1>{}, k + 1);
         half = 2 * W - half;
         if (MODE == Pass::Diag && ((k & 6) == 6 || k + 2 >= iters)) {
-            acc.r += sum_r.take();
-            acc.b += sum_b.take();
-            acc.jx += sum_jx.take();
-            acc.jy += sum_jy.take();
+            sum_mass.take(acc.r, acc.b);
+            sum_mom.take(acc.jx, acc.jy);
         }
     }
     if (MODE == Pass::Diag)
