@@ -362,8 +362,8 @@ cmrt_status cmrt_batch_step(cmrt_batch* b, int64_t n);
  * events) that read the current state and write the other buffer, so the
  * state does not advance.  cache_path (may be NULL): a JSON array, one
  * object per line, keyed by device name, SM count and the batch signature
- * (precision, vector path, size classes with their counts); a matching
- * entry is applied without measuring unless flags has CMRT_TUNE_FORCE, and
+ * (revision of the batched kernel, precision, vector path, strip window,
+ * size classes with their counts); a matching entry is applied without measuring unless flags has CMRT_TUNE_FORCE, and
  * a measurement replaces it.  us_per_step (may be NULL) receives the best
  * time of one batched step in microseconds (the cached one on a hit). */
 cmrt_status cmrt_batch_tune(cmrt_batch* b, const char* cache_path, int32_t flags, double* us_per_step);

@@ -1273,12 +1273,13 @@ bool parse_rows(const std::string& s, std::map<std::string, int>& rows) {
     return true;
 }
 
-// Signature of what the tuned rows depend on: storage, vector path and the
-// multiset of size classes.
+// Signature of what the tuned rows and their time depend on: the kernel's revision,
+// storage, vector path, strip window and the multiset of size classes.
 std::string batch_signature(const Batch* b) {
     std::map<std::string, int> count;
     for (const cmrt_params& p : b->p) count[class_key(p)]++;
-    std::string s = "p" + std::to_string(b->precision) + " v" + std::to_string(b->vec ? 1 : 0);
+    std::string s = "k" + std::to_string(cmrt::kBatchRevision) + " p" + std::to_string(b->precision) + " v" +
+                    std::to_string(b->vec ? 1 : 0) + " c" + std::to_string(b->window);
     for (const auto& kv : count) s += " " + kv.first + "*" + std::to_string(kv.second);
     return s;
 }

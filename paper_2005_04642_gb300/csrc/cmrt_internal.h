@@ -161,6 +161,10 @@ struct BatchArgs {
     unsigned* counters;         // [2] next item, CTAs finished; zero between launches
 };
 
+// Raised with every change of the batched kernel that moves its times: rows tuned on
+// another revision are measured anew.
+constexpr int kBatchRevision = 2;
+
 // What the batched kernel is compiled for: storage, 16-byte copies (every nx a
 // multiple of 4), whether any member has walls, and the columns of a strip's
 // window (96 or kWin, of which all but 2 kHalo are the strip's own).

@@ -157,6 +157,29 @@ def test_tuner_keeps_state_and_uses_cache(tmp_path):
         x.close()
 
 
+def test_tuner_ignores_rows_measured_on_another_kernel(tmp_path):
+    """A cache written before the batched kernel's strips and pipeline changed
+    (no strip width or kernel revision in its signature) is measured anew."""
+    members = _mixed_members(seed=16)
+    count = {}
+    for d, _, _ in members:
+        key = f"{d['nx']}x{d['ny']}w{int(bool(d['wall_y']))}"
+        count[key] = count.get(key, 0) + 1
+    vec = int(all(d["nx"] % 4 == 0 for d, _, _ in members))
+    sig = " ".join([f"p0 v{vec}"] + [f"{k}*{n}" for k, n in sorted(count.items())])
+    prop = torch.cuda.get_device_properties(0)
+    rows = " ".join(f"{k}=1" for k in sorted(count))
+    cache = tmp_path / "tune.json"
+    cache.write_text(f'[\n{{"device": "{prop.name}", "sms": {prop.multi_processor_count}, "signature": "{sig}", '
+                     f'"rows": "{rows}", "us_per_step": 12345.0}}\n]\n')
+    b = cm.Batch(members)
+    n0 = b.launches
+    us = b.tune(str(cache))
+    assert b.launches > n0 and us != 12345.0
+    assert cache.read_text().count('"signature"') == 2  # the other kernel's entry stays
+    b.close()
+
+
 def test_member_views():
     members = _mixed_members(seed=14)[:3]
     b = cm.Batch(members)
