@@ -39,8 +39,8 @@ BYTES_PER_CELL = 144  # 18 FP32 populations read + 18 written per node update
 N_SIDE = 8192
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal (the roofline uses the measured copy bandwidth)
 WORKLOAD = "drops_8192x8192_periodic_64drops_Lambda10"
-KERNEL_SOURCES = ["paper_2005_04642_gb300/csrc/cmrt_march.cuh", "paper_2005_04642_gb300/csrc/cmrt_device.cuh",
-                  "paper_2005_04642_gb300/csrc/cmrt_internal.h"]
+KERNEL_SOURCES = ["paper_2005_04642_gb300/csrc/cmrt_march.cuh", "paper_2005_04642_gb300/csrc/cmrt_step.cu",
+                  "paper_2005_04642_gb300/csrc/cmrt_device.cuh", "paper_2005_04642_gb300/csrc/cmrt_internal.h"]
 
 
 def workload_config(side=N_SIDE):

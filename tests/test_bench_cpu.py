@@ -33,6 +33,14 @@ def test_committed_traffic_summary_names_its_kernel_source():
     assert os.path.exists(os.path.join(REPO, d["summary"]))
 
 
+def test_kernel_sources_hold_what_sets_the_steps_traffic():
+    """The kernel, its building blocks and the rule for its rows per CTA (which
+    sets the fill rows each CTA reads again)."""
+    text = "".join(open(os.path.join(REPO, rel)).read() for rel in bench.KERNEL_SOURCES)
+    for definition in ("k_march(const char*", "\nint chain_rows(", "collide_increment(const float", "struct StepParams {"):
+        assert definition in text, definition
+
+
 def test_traffic_is_reported_only_for_the_source_it_was_taken_on(tmp_path, monkeypatch):
     monkeypatch.setattr(bench, "ROOT", str(tmp_path))
     _tree(tmp_path, {"source_sha": "0" * 16, "dram_bytes_per_cell": 145.0})
