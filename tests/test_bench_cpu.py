@@ -37,7 +37,7 @@ def test_kernel_sources_hold_what_sets_the_steps_traffic():
     """The kernel, its building blocks and the rule for its rows per CTA (which
     sets the fill rows each CTA reads again)."""
     text = "".join(open(os.path.join(REPO, rel)).read() for rel in bench.KERNEL_SOURCES)
-    for definition in ("k_march(const char*", "\nint chain_rows(", "collide_increment(const float", "struct StepParams {"):
+    for definition in ("k_march(const char*", "int chain_rows(int nx, int ny, int sms, int precision) {", "collide_increment(const float", "struct StepParams {"):
         assert definition in text, definition
 
 
