@@ -1091,17 +1091,23 @@ dim3 small_grid(const StepParams& P, int H) {
     return dim3(static_cast<unsigned>((P.nx + tx - 1) / tx), static_cast<unsigned>((P.ny + ty - 1) / ty));
 }
 
-// Whether a step runs as k_small.  FP32, per step with 16 window rows: 18.3,
-// 22.4, 29.7 and 40.4 us at 640^2, 720^2, 800^2 and 900^2, whatever the width;
-// the march 21.2, 22.4, 25.9 and 27.3 us with 16-byte copies; at 801^2 and 901^2,
-// with 4-byte ones (nx not a multiple of 4), 29.6 and 33.2 us.  16-bit: 16.7, 24.5
-// and 29.9 us at 512^2, 640^2 and 720^2 against the march's 18.8, 24.4 and 30.7.
+// Whether a step runs as k_small: up to where the march, whose copies are of 4
+// bytes where nx is no multiple of 4, becomes the faster on average.  Per step,
+// k_small against the march:
+//   FP32, 16-byte copies: 640^2 18.3 and 19.4 us, 700^2 21.4 and 20.5, 1024 x 512
+//     22.8 and 23.0, 256 x 2048 22.6 and 25.5, 736^2 24.1 and 22.2, 776 x 772 26.9
+//     and 21.9;
+//   FP32, 4-byte: 653^2 19.4 and 20.9, 721^2 22.7 and 24.2, 763^2 26.0 and 25.6, 491
+//     x 1201 26.1 and 27.6, 775^2 27.0 and 26.4, 801^2 29.8 and 26.5, 837^2 34.0 and 28.6;
+//   FP16, 16-byte: 512^2 16.7 and 17.8, 540^2 18.5 and 17.7, 1024 x 300 18.6 and
+//     19.3, 576^2 19.7 and 19.1, 640^2 24.3 and 23.1;
+//   FP16, 4-byte: 575^2 20.4 and 21.7, 601^2 23.0 and 26.1, 655^2 26.6 and 27.3.
 template <class L>
 bool use_small(const StepParams& P) {
-    const long nodes = static_cast<long>(P.nx) * P.ny;
-    const long limit = L::kDecode ? 330000 : 600000;
+    const bool vec = (P.nx % 4) == 0;
+    const long limit = L::kDecode ? (vec ? 330000 : 430000) : (vec ? 530000 : 600000);
     const int rows = 16 - 2 * small_halo<L>();
-    return nodes <= ((P.nx % 4) == 0 ? limit : limit + 100000) && P.ny <= 65535 * rows;  // grid rows
+    return static_cast<long>(P.nx) * P.ny <= limit && P.ny <= 65535 * rows;  // grid rows
 }
 
 // Window rows of k_small: a step takes about 1.7 us plus c ceil(tiles / SMs),
