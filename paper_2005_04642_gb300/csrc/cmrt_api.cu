@@ -128,7 +128,7 @@ struct Batch {
     cmrt::BatchItem* d_items = nullptr;
     size_t items_cap = 0;
     int nitems = 0;
-    int grid = 0;                        // persistent CTAs
+    int grid = 0;                        // persistent CTAs that fit on the GPU
     int window = cmrt::kWin;             // columns of a strip's window
     int tile() const { return window - 2 * cmrt::kHalo; }
     cmrt::BatchForm form() const { return {precision, vec, walls, window}; }
@@ -1169,7 +1169,10 @@ cudaError_t batch_launch(Batch* b, int src_parity, cudaStream_t s) {
     cmrt::BatchArgs A{b->d_items, b->nitems, b->d_params, b->d_off,
                       static_cast<const char*>(b->buf[src_parity]), static_cast<char*>(b->buf[src_parity ^ 1]),
                       b->d_flags, b->d_counters};
-    return cmrt::launch_batch(A, b->form(), b->grid, s);
+    // no more CTAs than items: surplus ones would leave the hardware's spread over the
+    // SMs to which CTAs reach the counter first (152 items of 41 x 512: 1127 us per
+    // step, several items on some SMs and none on others; 638 us spread)
+    return cmrt::launch_batch(A, b->form(), std::min(b->grid, b->nitems), s);
 }
 
 // Records graph_steps batched steps starting from buffer parity `parity`.

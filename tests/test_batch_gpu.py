@@ -180,6 +180,32 @@ def test_tuner_ignores_rows_measured_on_another_kernel(tmp_path):
     b.close()
 
 
+def test_few_items_spread_over_the_gpu():
+    """A batch of one work item per SM leaves none of them idle: its step takes
+    clearly less time than one of four such items per SM (one column strip each,
+    16-byte copies ruled out; 0.99 of it when CTAs took items in the order they
+    started)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    d = I.base_params(41, 256)
+    times = []
+    for n in (sms, 4 * sms):
+        b = cm.Batch([(d, None, None)] * n)
+        b.set_rows(41, 256, 0, 256)
+        assert b.work_items == n
+        b.step(32)
+        best = float("inf")
+        for _ in range(5):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            b.step(32)
+            e1.record()
+            e1.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        times.append(best)
+        b.close()
+    assert times[0] <= 0.75 * times[1], times
+
+
 def test_member_views():
     members = _mixed_members(seed=14)[:3]
     b = cm.Batch(members)
