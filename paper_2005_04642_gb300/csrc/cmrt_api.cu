@@ -1061,9 +1061,6 @@ std::string class_key(const cmrt_params& p) {
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
-// Rows per work item before tuning: whole lattices up to 64 rows, else 64.
-int default_rows(const cmrt_params& p) { return std::min(64, std::max(1, p.ny)); }
-
 // Window width of a batch: strips of 88 or of 120 own columns, whichever
 // computes fewer window columns over all members.  512 and 256 columns take 6
 // and 3 windows of 96 (576 and 288 columns) against 5 and 3 of 128 (640 and
@@ -1077,6 +1074,40 @@ int batch_window(const std::vector<cmrt_params>& ps) {
             cols[k] += static_cast<double>((p.nx + tile - 1) / tile) * width[k] * p.ny;
         }
     return cols[0] < cols[1] ? width[0] : width[1];
+}
+
+// Rows per work item before tuning (whole lattices up to that): 64, or where the
+// GPU holds all items of some shorter or longer rows at once, those of them that take
+// the least time: the longest item's rows + 7 iterations (7 fill the pipeline) on
+// the fullest SM, where an iteration takes, measured, 1, 1.17, 1.3, 1.42 and 1.68
+// times as long with one to five CTAs of 96 columns, 1, 1.22, 1.5 and 1.9 with one
+// to four of 128.  With 64 rows throughout, 96 members of 24^2 .. 48^2 took 68 us
+// per step (33 with this rule), 16 of 64^2 .. 512^2 79 (50), 96 of 8 and 17 x 600
+// 240 (224).  Longer lists keep 64: what a model of whole and part rounds of items
+// chose was slower as often as faster (96 members of 64 .. 512 columns: 272 against
+// 256 us, 307 against 287).
+int default_rows(const Batch* b, int sms) {
+    constexpr double kIter[2][5] = {{1.0, 1.17, 1.3, 1.42, 1.68}, {1.0, 1.22, 1.5, 1.9, 1.9}};
+    constexpr int kFill = 7;
+    const int full = std::min(5, b->grid / sms);
+    int best = 64;
+    double best_time = 1e30;
+    for (const int rows : {16, 24, 32, 48, 64, 96}) {
+        int64_t items = 0;
+        int longest = 0;
+        for (const cmrt_params& p : b->p) {
+            items += static_cast<int64_t>((p.nx + b->tile() - 1) / b->tile()) * ((p.ny + rows - 1) / rows);
+            longest = std::max(longest, std::min(rows, p.ny));
+        }
+        if (items > b->grid) continue;
+        const int per_sm = std::min(full, static_cast<int>((items + sms - 1) / sms));
+        const double time = (longest + kFill) * kIter[b->window == cmrt::kWin][per_sm - 1];
+        if (time < best_time) {
+            best_time = time;
+            best = rows;
+        }
+    }
+    return best;
 }
 
 Batch* blive(cmrt_batch* h) {
@@ -1331,7 +1362,6 @@ cmrt_status cmrt_batch_init(int32_t n, const cmrt_params* params, const float* c
         b->off.push_back(b->arena_bytes);
         const size_t bytes = static_cast<size_t>(params[m].nx) * params[m].ny * node;
         b->arena_bytes += (bytes + 255) / 256 * 256;  // 256-byte aligned members
-        b->rows[class_key(params[m])] = default_rows(params[m]);
         if (params[m].diag_every > 0 && (b->diag_every == 0 || params[m].diag_every < b->diag_every))
             b->diag_every = params[m].diag_every;
     }
@@ -1375,6 +1405,8 @@ cmrt_status cmrt_batch_init(int32_t n, const cmrt_params* params, const float* c
         return bail(CMRT_ECUDA);
     }
     b->grid = per_sm * sms;
+    const int rows = default_rows(b, sms);
+    for (const cmrt_params& p : b->p) b->rows[class_key(p)] = std::min(rows, p.ny);
     // initial states, member by member, through the single-lattice path
     for (int m = 0; m < n; ++m) {
         Ctx tmp;

@@ -206,6 +206,15 @@ def test_few_items_spread_over_the_gpu():
     assert times[0] <= 0.75 * times[1], times
 
 
+@pytest.mark.parametrize("n,nx,ny,rows", [(96, 48, 48, range(1, 48)), (16, 256, 256, range(1, 64)), (48, 1024, 512, [64])])
+def test_default_rows_fill_the_gpu(n, nx, ny, rows):
+    """A batch too small to fill the GPU with 64 rows per item starts with shorter
+    segments, a large one with 64."""
+    b = cm.Batch([(I.base_params(nx, ny), None, None)] * n)
+    assert b.get_rows(nx, ny) in rows
+    b.close()
+
+
 def test_member_views():
     members = _mixed_members(seed=14)[:3]
     b = cm.Batch(members)
