@@ -104,12 +104,13 @@ __device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& e) {
     return s;
 }
 
-// A running pair of sums of up to eight FP32 terms in three FP32 parts: hi takes the
-// terms, mid the exact rests of its additions, lo the exact rests of mid's.  Only lo's
-// own additions round: with S the sum of the terms' magnitudes, mid stays below
-// 2^-21 S, lo below 2^-42 S and its error below 2^-63 S, so that the sums that take()
-// adds to FP64 accumulators are rounded there alone, less often than by an FP64
-// addition per term.  GB300's FP64 unit takes an SM 16 cycles per warp
+// A running pair of sums of FP32 terms in three FP32 parts: hi takes the terms, mid
+// the exact rests of its additions, lo the exact rests of mid's.  Only lo's own
+// additions round: of n terms with S the sum of their magnitudes, mid stays below
+// n 2^-24 S, lo below n^2 2^-48 S and its error below n^3 2^-72 S (2^-63 S of eight
+// terms, 2^-57 S of 32), so that the sums that take() adds to FP64 accumulators are
+// rounded there alone, less often than by an FP64 addition per term.  (Terms of 1e30
+// and more are the caller's to add in FP64.)  GB300's FP64 unit takes an SM 16 cycles per warp
 // instruction: a conversion and an addition per term bounded the diagnostics pass
 // (a call on 2048^2 154 us, on 8192 x 4096 1038; with Sum3 115 and 661; with hi
 // and lo alone, whose rest rounds at 2^-46 of the terms, 109 and 619).
@@ -125,6 +126,34 @@ struct Sum3 {
         x += static_cast<double>(hi.x) + (static_cast<double>(mid.x) + static_cast<double>(lo.x));
         y += static_cast<double>(hi.y) + (static_cast<double>(mid.y) + static_cast<double>(lo.y));
         hi = mid = lo = make_float2(0.0f, 0.0f);
+    }
+};
+
+// The fastest of a thread's nodes, to FP64's precision: |u|^2 as an FP32 pair, good to
+// 2^-46, decides, and the FP64 value of the node it chose counts; of nodes closer than
+// the pairs can tell (2^-42), or beyond the range in which a pair is that good, each
+// one's FP64 value goes to u2.
+struct Fastest {
+    float hi = 0.0f, lo = 0.0f, x = 0.0f, y = 0.0f;
+    __device__ __forceinline__ void add(float ux, float uy, double& u2) {
+        const float p = __fmul_rn(ux, ux), q = __fmul_rn(uy, uy);
+        float e;
+        const float s = two_sum(p, q, e);
+        const float low = e + (__fmaf_rn(ux, ux, -p) + __fmaf_rn(uy, uy, -q));
+        const float top = __fadd_rn(s, low), rest = low - (top - s);
+        const bool usual = top > 1e-28f && top < 1e30f;
+        const float lead = (top - hi) + (rest - lo), near = 0x1p-42f * top;
+        if (usual && lead > near) {
+            hi = top;
+            lo = rest;
+            x = ux;
+            y = uy;
+        } else if (usual ? lead >= -near && (ux != x || uy != y) : ux != 0.0f || uy != 0.0f) {
+            u2 = fmax(u2, static_cast<double>(ux) * ux + static_cast<double>(uy) * uy);
+        }
+    }
+    __device__ __forceinline__ void take(double& u2) const {
+        u2 = fmax(u2, static_cast<double>(x) * x + static_cast<double>(y) * y);
     }
 };
 

@@ -575,7 +575,7 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
 
     // diagnostics: up to eight rows' sums, and the fastest node so far
     Sum3 sum_mass, sum_mom;
-    float best_hi = 0.0f, best_lo = 0.0f, best_ux = 0.0f, best_uy = 0.0f;
+    Fastest fastest;
     // what the later stages of this column need.  f, rho_R, rho_B and j: before an
     // even iteration slots 0 .. 3 hold rows r - 1 .. r - 4, before an odd one
     // slots 1, 0, 3, 2; grad rho^N and G alternate
@@ -645,23 +645,7 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
                         acc.jx += mx;
                         acc.jy += my;
                     }
-                    // |u|^2 as an FP32 pair, good to 2^-46, finds the fastest node, whose FP64
-                    // value counts; of nodes closer than the pairs can tell (2^-42) each does
-                    const float p = __fmul_rn(ux, ux), q = __fmul_rn(uy, uy);
-                    float e;
-                    const float s = two_sum(p, q, e);
-                    const float lo = e + (__fmaf_rn(ux, ux, -p) + __fmaf_rn(uy, uy, -q));
-                    const float top = __fadd_rn(s, lo), rest = lo - (top - s);
-                    const bool usual = top > 1e-28f && top < 1e30f;
-                    const float lead = (top - best_hi) + (rest - best_lo), near = 0x1p-42f * top;
-                    if (usual && lead > near) {
-                        best_hi = top;
-                        best_lo = rest;
-                        best_ux = ux;
-                        best_uy = uy;
-                    } else if (usual ? lead >= -near && (ux != best_ux || uy != best_uy) : ux != 0.0f || uy != 0.0f) {
-                        acc.u2 = fmax(acc.u2, static_cast<double>(ux) * ux + static_cast<double>(uy) * uy);
-                    }
+                    fastest.add(ux, uy, acc.u2);
                 } else {
                     acc.bad += 1.0;
                 }
@@ -822,8 +806,7 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
             sum_mom.take(acc.jx, acc.jy);
         }
     }
-    if (MODE == Pass::Diag)
-        acc.u2 = fmax(acc.u2, static_cast<double>(best_ux) * best_ux + static_cast<double>(best_uy) * best_uy);
+    if (MODE == Pass::Diag) fastest.take(acc.u2);
     cp_wait<0>();
 }
 

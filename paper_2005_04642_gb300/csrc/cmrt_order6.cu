@@ -189,36 +189,47 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
         if (fo.uy) fo.uy[o] = uy;
         if (fo.p) fo.p[o] = fmaf(P.cs2_r, rr, P.cs2_b * rb);
     } else {
-        // FP64 partial diagnostics of the CTA (slot 4 is a maximum)
-        double v[kDiagSlots] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        if (own) {
-            if (isfinite(rho)) {
-                v[0] = rr;
-                v[1] = rb;
-                v[2] = jx;
-                v[3] = jy;
-                v[4] = static_cast<double>(ux) * ux + static_cast<double>(uy) * uy;
-            } else {
-                v[5] = 1.0;
-            }
-        }
-        __shared__ double red[H][kDiagSlots];
+        // FP64 partial diagnostics of the CTA (slot 4 is a maximum): a warp per two sums and
+        // one for the fastest node, a lane per column, over values left in the place of
+        // fields that are read no more.  A warp's FP64 instruction takes the SM 16 cycles:
+        // six FP64 shuffle reductions in every warp took two thirds of the pass (4096^2
+        // 3790 us, this 1765)
+        const bool counts = own && isfinite(rho);
+        const float part[6] = {rr, rb, jx, jy, ux, uy};
 #pragma unroll
-        for (int j = 0; j < kDiagSlots; ++j)
+        for (int j = 0; j < 6; ++j) w[(j < 4 ? j : j + 1) * kN] = counts ? part[j] : 0.0f;
+        const int bad = __syncthreads_count(own && !counts);
+        double* out = partials + (static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * kDiagSlots;
+        for (int q = ty; q < 3; q += H) {
+            const float *a = sm + kX + (q < 2 ? 2 * q : kUx) * kN + tx, *b = a + kN;
+            double v = 0.0, v2 = 0.0;
+            if (q < 2) {
+                Sum3 sum;
+                for (int k = kEdge; k < H - kEdge; ++k) {
+                    const float c = a[k * kX], d = b[k * kX];
+                    if (fmaxf(fabsf(c), fabsf(d)) < 1e30f) {
+                        sum.add(c, d);
+                    } else {
+                        v += c;
+                        v2 += d;
+                    }
+                }
+                sum.take(v, v2);
+            } else {
+                Fastest fastest;
+                for (int k = kEdge; k < H - kEdge; ++k) fastest.add(a[k * kX], b[k * kX], v);
+                fastest.take(v);
+            }
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) {
-                const double u = __shfl_down_sync(0xffffffffu, v[j], off);
-                v[j] = j == 4 ? fmax(v[j], u) : v[j] + u;
+                const double u = __shfl_down_sync(0xffffffffu, v, off);
+                v = q == 2 ? fmax(v, u) : v + u;
+                if (q < 2) v2 += __shfl_down_sync(0xffffffffu, v2, off);
             }
-        if (tx == 0)
-#pragma unroll
-            for (int j = 0; j < kDiagSlots; ++j) red[ty][j] = v[j];
-        __syncthreads();
-        if (threadIdx.x < kDiagSlots) {
-            double acc = 0.0;
-            for (int k = kEdge; k < H - kEdge; ++k)
-                acc = threadIdx.x == 4 ? fmax(acc, red[k][threadIdx.x]) : acc + red[k][threadIdx.x];
-            partials[(static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * kDiagSlots + threadIdx.x] = acc;
+            if (tx == 0) {
+                out[2 * q] = v;
+                out[2 * q + 1] = q < 2 ? v2 : static_cast<double>(bad);
+            }
         }
     }
 }

@@ -26,8 +26,8 @@ cm.load()
 NX, NY = 4, 8192  # a column of many rows per CTA
 
 
-def _lattice():
-    return cm.Lattice(I.base_params(NX, NY), None, None)
+def _lattice(order):
+    return cm.Lattice(I.base_params(NX, NY, stencil_order=order), None, None)
 
 
 def _state():
@@ -42,12 +42,13 @@ TERMS = np.array([2.4680748555994114e-09, -0.13798120617866516, 1.62853598340007
                  np.float32)
 
 
+@pytest.mark.parametrize("order", [2, 6])
 @pytest.mark.parametrize("axis", [0, 1], ids=["x", "y"])
-def test_momentum_of_terms_of_unequal_size(axis):
+def test_momentum_of_terms_of_unequal_size(axis, order):
     plus, minus = ((8, 4), (2, 6))[axis]
     want = math.fsum(TERMS.tolist())
     bound = 8 * 2.0**-53 * math.fsum(abs(v) for v in TERMS.tolist())
-    lat = _lattice()
+    lat = _lattice(order)
     for shift in range(16):  # wherever the rows of a CTA and its groups of rows begin
         pops = _state()
         for k, v in enumerate(TERMS):
@@ -64,9 +65,10 @@ CLOSE = [("0x1.d767840000000p-26", "0x1.3419520000000p-32", "0x1.d767860000000p-
          ("0x1.abfcea0000000p-26", "0x1.933d600000000p-33", "0x1.abfcec0000000p-26", "0x1.92b56e0000000p-33")]
 
 
+@pytest.mark.parametrize("order", [2, 6])
 @pytest.mark.parametrize("swap", [False, True])
 @pytest.mark.parametrize("pair", CLOSE, ids=["first_faster", "second_faster"])
-def test_fastest_of_two_nodes_of_nearly_one_speed(pair, swap):
+def test_fastest_of_two_nodes_of_nearly_one_speed(pair, swap, order):
     v = [float.fromhex(x) for x in pair]
     nodes = [(v[0], v[1]), (v[2], v[3])]
     want = max(math.sqrt(x * x + y * y) for x, y in nodes)
@@ -74,7 +76,7 @@ def test_fastest_of_two_nodes_of_nearly_one_speed(pair, swap):
     for k, (x, y) in enumerate(nodes[::-1] if swap else nodes):
         pops[0, 8, 201 + k, 1] = x
         pops[0, 2, 201 + k, 1] = y
-    lat = _lattice()
+    lat = _lattice(order)
     lat.set_populations(pops)
     f = lat.fields()
     assert sorted(f["ux"].unique().tolist()) == sorted({0.0, v[0], v[2]})  # u is the momentum
