@@ -23,7 +23,11 @@
 namespace cmrt {
 namespace {
 
-constexpr int kX = 32, kEdge = 5;
+constexpr int kX = 32;
+// halo of a window: 5 for the step; the fields and diagnostics end with u, which reads
+// populations up to 4 away (24 instead of 22 own columns and rows of 32: fields of
+// 4096^2 790 -> 680 us, diagnostics 1765 -> 1543)
+constexpr int edge_of(Pass mode) { return mode == Pass::Step ? 5 : 4; }
 
 __device__ __forceinline__ int wrap(int v, int n) {
     if (v >= 0 && v < n) return v;
@@ -44,7 +48,7 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
     k_order6(const float* __restrict__ src, float* __restrict__ dst, const StepParams P, FieldOut fo,
              unsigned* __restrict__ flag, double* __restrict__ partials) {
     pdl_begin();
-    constexpr int kN = kX * H;
+    constexpr int kN = kX * H, kEdge = edge_of(MODE);
     __shared__ float sm[7 * kN + 2 * kX];
     const int tx = threadIdx.x % kX, ty = threadIdx.x / kX;
     const int nx = P.nx, ny = P.ny;
@@ -234,22 +238,22 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
     }
 }
 
-dim3 grid6(int nx, int ny, int H) {
-    const int tx = kX - 2 * kEdge, ty = H - 2 * kEdge;
+dim3 grid6(int nx, int ny, int H, int edge) {
+    const int tx = kX - 2 * edge, ty = H - 2 * edge;
     return dim3(static_cast<unsigned>((nx + tx - 1) / tx), static_cast<unsigned>((ny + ty - 1) / ty));
 }
 
 // Window rows: 16 (two CTAs per SM) while that is at most two windows per SM, else 32.
-int rows6(int nx, int ny) {
-    const dim3 g = grid6(nx, ny, 16);
+int rows6(int nx, int ny, int edge) {
+    const dim3 g = grid6(nx, ny, 16, edge);
     return static_cast<long>(g.x) * g.y <= 304 ? 16 : 32;
 }
 
 template <Pass MODE>
 cudaError_t launch6(const float* src, float* dst, const StepParams& P, FieldOut fo, unsigned* flag, double* partials,
                     cudaStream_t s) {
-    const int H = rows6(P.nx, P.ny);
-    const dim3 g = grid6(P.nx, P.ny, H);
+    const int H = rows6(P.nx, P.ny, edge_of(MODE));
+    const dim3 g = grid6(P.nx, P.ny, H, edge_of(MODE));
     auto go = [&](auto k) { return launch_pdl(k, g, dim3(kX * H), 0, s, src, dst, P, fo, flag, partials); };
     if (H == 16) return P.wall_y ? go(&k_order6<16, true, MODE>) : go(&k_order6<16, false, MODE>);
     return P.wall_y ? go(&k_order6<32, true, MODE>) : go(&k_order6<32, false, MODE>);
@@ -264,7 +268,8 @@ cudaError_t launch_fields6(const float* src, const StepParams& P, FieldOut out, 
     return launch6<Pass::Fields>(src, nullptr, P, out, nullptr, nullptr, s);
 }
 int diag_blocks6(int nx, int ny) {
-    const dim3 g = grid6(nx, ny, rows6(nx, ny));
+    const int edge = edge_of(Pass::Diag);
+    const dim3 g = grid6(nx, ny, rows6(nx, ny, edge), edge);
     return static_cast<int>(g.x * g.y);
 }
 cudaError_t launch_diag6(const float* src, const StepParams& P, double* partials, cudaStream_t s) {
