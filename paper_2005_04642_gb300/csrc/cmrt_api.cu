@@ -612,7 +612,7 @@ cmrt_status cmrt_init(const cmrt_params* p, const float* rho_n0, const float* u0
     c->rows = cmrt::chain_rows(p->nx, p->ny, sms, p->precision);
     const dim3 g = cmrt::chain_grid(p->nx, p->ny, c->rows);
     c->n_partials = static_cast<int>(g.x * g.y);
-    if (p->stencil_order == 6) c->n_partials = cmrt::diag_blocks6(p->nx, p->ny);
+    if (p->stencil_order == 6) c->n_partials = cmrt::diag_blocks6(c->sp);
     if (cudaMalloc(&c->d_flag, sizeof(unsigned)) != cudaSuccess ||
         cudaMalloc(&c->d_partials, sizeof(double) * cmrt::kDiagSlots * c->n_partials) != cudaSuccess ||
         cudaMalloc(&c->d_diag, sizeof(double) * cmrt::kDiagSlots) != cudaSuccess) {

@@ -184,7 +184,7 @@ cudaError_t launch_batch(const BatchArgs& A, const BatchForm& b, int grid, cudaS
 // partials[diag_blocks6][kDiagSlots].
 cudaError_t launch_step6(const float* src, float* dst, const StepParams& P, unsigned* flag, cudaStream_t s);
 cudaError_t launch_fields6(const float* src, const StepParams& P, FieldOut out, cudaStream_t s);
-int diag_blocks6(int nx, int ny);
+int diag_blocks6(const StepParams& P);
 cudaError_t launch_diag6(const float* src, const StepParams& P, double* partials, cudaStream_t s);
 
 // Discrete adjoint (cmrt_planes.cu), FP32 storage.  scratch: float[kAdjPlanes][ny][nx];

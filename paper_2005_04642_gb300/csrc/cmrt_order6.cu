@@ -4,7 +4,7 @@
 // a stencil of radius 3, with the compact one for K and div u.
 //
 // One node per thread: a CTA takes a window of 32 x H nodes, 22 x (H - 10) of
-// them its own, gathers each node's populations into registers and runs
+// them its own (all H rows of a lattice of at most 32), gathers each node's populations into registers and runs
 //   moments, chi, Phi' | grad rho^N (halo 2) | K, G, u (halo 1) | the rest,
 // with a barrier between, the fields that a stencil reads in shared memory.
 // What bounds it: the launch and one load latency on small lattices, else
@@ -23,9 +23,9 @@
 namespace cmrt {
 namespace {
 
-constexpr int kX = 32;
-// halo of a window: 5 for the step; the fields and diagnostics end with u, which reads
-// populations up to 4 away (24 instead of 22 own columns and rows of 32: fields of
+constexpr int kX = 32, kMaxRows = 32;
+// halo of a window: 5 for the step; the fields and diagnostics end with u, which needs
+// moments up to 4 away (24 instead of 22 own columns and rows of 32: fields of
 // 4096^2 790 -> 680 us, diagnostics 1765 -> 1543)
 constexpr int edge_of(Pass mode) { return mode == Pass::Step ? 5 : 4; }
 
@@ -43,22 +43,25 @@ __device__ __forceinline__ void normal_of(float gx, float gy, float& nx, float& 
 // App. B coefficients a_N
 __host__ __device__ constexpr float coef(int N) { return N == 1 ? 4.5f : (N == 2 ? -0.9f : 0.1f); }
 
-template <int H, bool W, Pass MODE>
-__global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
+// ROWS: the window's rows (0: those of the launch); FLAT: a window has the lattice's rows
+// and no others (ROWS 0)
+template <int ROWS, bool FLAT, bool W, Pass MODE>
+__global__ void __launch_bounds__(kX * kMaxRows, 1)
     k_order6(const float* __restrict__ src, float* __restrict__ dst, const StepParams P, FieldOut fo,
              unsigned* __restrict__ flag, double* __restrict__ partials) {
     pdl_begin();
-    constexpr int kN = kX * H, kEdge = edge_of(MODE);
-    __shared__ float sm[7 * kN + 2 * kX];
+    constexpr int kEdge = edge_of(MODE);
+    const int kN = ROWS ? kX * ROWS : static_cast<int>(blockDim.x), H = kN / kX;
+    extern __shared__ float sm[];
     const int tx = threadIdx.x % kX, ty = threadIdx.x / kX;
     const int nx = P.nx, ny = P.ny;
     const size_t nodes = static_cast<size_t>(nx) * ny;
     const int xw = static_cast<int>(blockIdx.x) * (kX - 2 * kEdge) - kEdge + tx;
     const int yw = static_cast<int>(blockIdx.y) * (H - 2 * kEdge) - kEdge + ty;
-    const int x = wrap(xw, nx), y = W ? yw : wrap(yw, ny);
-    const bool in = !W || (y >= 0 && y < ny);
-    auto inner = [&](int d) { return in && tx >= d && tx < kX - d && ty >= d && ty < H - d; };
-    const bool own = inner(kEdge) && xw < nx && yw < ny;
+    const int x = wrap(xw, nx), y = FLAT ? ty : W ? yw : wrap(yw, ny);
+    const bool in = FLAT || !W || (y >= 0 && y < ny);
+    auto inner = [&](int d) { return in && tx >= d && tx < kX - d && (FLAT || (ty >= d && ty < H - d)); };
+    const bool own = inner(kEdge) && xw < nx && (FLAT || yw < ny);
     const bool low = W && y == 0, high = W && y == ny - 1;
     float* w = sm + kX + threadIdx.x;  // this node in a field of the window
     constexpr int kChiR = 0, kChiB = 1, kPhi = 2, kGx = 3, kGy = 4, kUx = 5, kUy = 6;
@@ -67,7 +70,8 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
         int t = y + dy;
         if (W && t < 0) t = -1 - t;
         if (W && t >= ny) t = 2 * ny - 1 - t;
-        return W ? (t - y) * kX : dy * kX;
+        if (FLAT && !W) t = wrap(t, ny);
+        return W || FLAT ? (t - y) * kX : dy * kX;
     };
     auto grad6 = [&](const float* a, float& gx, float& gy) {
         gx = 0.0f;
@@ -84,7 +88,7 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
         }
     };
     // compact derivatives: beyond a wall the node's own row times the field's parity
-    const int up = high ? 0 : kX, dn = low ? 0 : -kX;
+    const int up = FLAT && !W ? row(1) : high ? 0 : kX, dn = FLAT && !W ? row(-1) : low ? 0 : -kX;
     auto d_x = [&](const float* a, float parity) {
         const float pu = high ? parity : 1.0f, pd = low ? parity : 1.0f;
         return ddx(a[1], a[-1], pu * a[up + 1], pu * a[up - 1], pd * a[dn + 1], pd * a[dn - 1]);
@@ -204,12 +208,13 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
         for (int j = 0; j < 6; ++j) w[(j < 4 ? j : j + 1) * kN] = counts ? part[j] : 0.0f;
         const int bad = __syncthreads_count(own && !counts);
         double* out = partials + (static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * kDiagSlots;
+        const int first = FLAT ? 0 : kEdge;
         for (int q = ty; q < 3; q += H) {
             const float *a = sm + kX + (q < 2 ? 2 * q : kUx) * kN + tx, *b = a + kN;
             double v = 0.0, v2 = 0.0;
             if (q < 2) {
                 Sum3 sum;
-                for (int k = kEdge; k < H - kEdge; ++k) {
+                for (int k = first; k < H - first; ++k) {
                     const float c = a[k * kX], d = b[k * kX];
                     if (fmaxf(fabsf(c), fabsf(d)) < 1e30f) {
                         sum.add(c, d);
@@ -221,7 +226,7 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
                 sum.take(v, v2);
             } else {
                 Fastest fastest;
-                for (int k = kEdge; k < H - kEdge; ++k) fastest.add(a[k * kX], b[k * kX], v);
+                for (int k = first; k < H - first; ++k) fastest.add(a[k * kX], b[k * kX], v);
                 fastest.take(v);
             }
 #pragma unroll
@@ -238,25 +243,45 @@ __global__ void __launch_bounds__(kX * H, 1024 / (kX * H))
     }
 }
 
+// Lattices of at most 32 rows are one window high, without halo rows: the row beyond
+// an edge, periodic or mirrored, is a row of the window.  150000 x 4: 30 us per step
+// with 4 window rows, 148 with 32 of which 22 own (45 as plane passes); 20000 x 24: 30
+// against 48 (35).
+bool flat6(int ny) { return ny <= kMaxRows; }
+
 dim3 grid6(int nx, int ny, int H, int edge) {
     const int tx = kX - 2 * edge, ty = H - 2 * edge;
-    return dim3(static_cast<unsigned>((nx + tx - 1) / tx), static_cast<unsigned>((ny + ty - 1) / ty));
+    return dim3(static_cast<unsigned>((nx + tx - 1) / tx), flat6(ny) ? 1u : static_cast<unsigned>((ny + ty - 1) / ty));
 }
 
-// Window rows: 16 (two CTAs per SM) while that is at most two windows per SM, else 32.
-int rows6(int nx, int ny, int edge) {
-    const dim3 g = grid6(nx, ny, 16, edge);
-    return static_cast<long>(g.x) * g.y <= 304 ? 16 : 32;
+// Window rows: the lattice's where it is flat; else 16 (two CTAs per SM) while that is
+// at most two windows per SM, else 32, or those of 17 to 31 of a periodic lattice that
+// save at least 4 % of the rows computed (rows known only at the launch cost 1 to 2 %;
+// halo rows beyond a wall are idle anyway).  20000 x 33: 56 us per step with 32 rows,
+// 52 with 27.
+int rows6(const StepParams& P, int edge) {
+    if (flat6(P.ny)) return P.ny;
+    const dim3 g = grid6(P.nx, P.ny, 16, edge);
+    if (static_cast<long>(g.x) * g.y <= 304) return 16;
+    int best = kMaxRows;
+    auto computed = [&](int H) { return static_cast<long>((P.ny + H - 2 * edge - 1) / (H - 2 * edge)) * H; };
+    for (int H = kMaxRows - 1; H > 16 && !P.wall_y; --H)
+        if (computed(H) < computed(best) && computed(H) * 100 <= computed(kMaxRows) * 96) best = H;
+    return best;
 }
 
 template <Pass MODE>
 cudaError_t launch6(const float* src, float* dst, const StepParams& P, FieldOut fo, unsigned* flag, double* partials,
                     cudaStream_t s) {
-    const int H = rows6(P.nx, P.ny, edge_of(MODE));
+    const int H = rows6(P, edge_of(MODE));
     const dim3 g = grid6(P.nx, P.ny, H, edge_of(MODE));
-    auto go = [&](auto k) { return launch_pdl(k, g, dim3(kX * H), 0, s, src, dst, P, fo, flag, partials); };
-    if (H == 16) return P.wall_y ? go(&k_order6<16, true, MODE>) : go(&k_order6<16, false, MODE>);
-    return P.wall_y ? go(&k_order6<32, true, MODE>) : go(&k_order6<32, false, MODE>);
+    auto go = [&](auto k) {
+        return launch_pdl(k, g, dim3(kX * H), (7 * kX * H + 2 * kX) * sizeof(float), s, src, dst, P, fo, flag, partials);
+    };
+    if (flat6(P.ny)) return P.wall_y ? go(&k_order6<0, true, true, MODE>) : go(&k_order6<0, true, false, MODE>);
+    if (H == 16) return P.wall_y ? go(&k_order6<16, false, true, MODE>) : go(&k_order6<16, false, false, MODE>);
+    if (H == 32) return P.wall_y ? go(&k_order6<32, false, true, MODE>) : go(&k_order6<32, false, false, MODE>);
+    return go(&k_order6<0, false, false, MODE>);
 }
 
 }  // namespace
@@ -267,9 +292,8 @@ cudaError_t launch_step6(const float* src, float* dst, const StepParams& P, unsi
 cudaError_t launch_fields6(const float* src, const StepParams& P, FieldOut out, cudaStream_t s) {
     return launch6<Pass::Fields>(src, nullptr, P, out, nullptr, nullptr, s);
 }
-int diag_blocks6(int nx, int ny) {
-    const int edge = edge_of(Pass::Diag);
-    const dim3 g = grid6(nx, ny, rows6(nx, ny, edge), edge);
+int diag_blocks6(const StepParams& P) {
+    const dim3 g = grid6(P.nx, P.ny, rows6(P, edge_of(Pass::Diag)), edge_of(Pass::Diag));
     return static_cast<int>(g.x * g.y);
 }
 cudaError_t launch_diag6(const float* src, const StepParams& P, double* partials, cudaStream_t s) {

@@ -150,3 +150,36 @@ def test_batches_with_16_byte_copies_give_the_bits_of_windows(shapes, walls, pre
         assert torch.equal(b.member(k).populations(), lat.populations()), (m[0]["nx"], m[0]["ny"])
         lat.close()
     b.close()
+
+
+# App. B's stencil: lattices of one window's height (periodic rows that wrap inside
+# it, walls), window heights chosen for the lattice's (33 and 40 rows), 22 and 24
+# own columns
+@pytest.mark.parametrize("nx,ny,wall", [(25, 1, False), (30, 2, False), (44, 3, True), (23, 5, False), (67, 31, True),
+                                        (45, 32, False), (24, 32, True), (1900, 33, False), (1900, 40, False)])
+def test_order6_windows_of_low_lattices_match_oracle(nx, ny, wall):
+    d = I.base_params(nx, ny, wall_y=wall, g_acc=(1e-5, -2e-5), stencil_order=6)
+    y, x = np.mgrid[0:ny, 0:nx]
+    rn = np.tanh(3.0 * np.sin(2 * np.pi * x / nx + 0.3) * (1.0 if ny < 8 else np.cos(np.pi * y / ny) + 0.4))
+    u = I.velocity_noise(nx, ny, 0.01, 7)
+    lat = cm.Lattice(d, rn.astype(np.float32), u.astype(np.float32))
+    lat.step(3)
+    got = lat.populations().double().cpu().numpy()
+    p = O.Params(**d)
+    R, B = O.init_state(rn.astype(np.float32).astype(np.float64), *u.astype(np.float32).astype(np.float64), p)
+    R, B = O.run(R, B, p, 3)
+    ref = np.stack([R, B])
+    assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max()
+    f, got = lat.fields(), lat.diagnostics()
+    assert got["mass_r"] == pytest.approx(R.sum(), rel=2e-6) and got["mass_b"] == pytest.approx(B.sum(), rel=2e-6)
+    assert got["umax"] == pytest.approx(float(torch.hypot(f["ux"].double(), f["uy"].double()).max()), rel=1e-6)
+    if not wall:
+        # the same rows again and again, on a lattice of windows with halo rows: the same bits
+        k = 66 // ny + 1
+        tall = cm.Lattice(dict(d, ny=k * ny), np.tile(rn, (k, 1)).astype(np.float32), np.tile(u, (1, k, 1)).astype(np.float32))
+        tall.step(3)
+        assert torch.equal(tall.populations(), lat.populations().tile(1, 1, k, 1))
+        for name, v in tall.fields().items():
+            assert torch.equal(v, f[name].tile(k, 1)), name
+        tall.close()
+    lat.close()
