@@ -323,8 +323,8 @@ const char* cmrt_last_error(const cmrt_ctx* c);
  * facility for running many independent lattices of uneven sizes, each the
  * scheme above with its own parameters (sigma, Lambda, alpha, relaxation
  * rates, forces, walls), in ONE persistent kernel launch per time step.  The
- * launch drains a work list of tiles (member, 120-column strip, segment of
- * rows), longest segments first; no CTA ever waits on another, so there is
+ * launch drains a work list of tiles (member, strip of 88 or 120 columns,
+ * segment of rows), longest segments first; no CTA ever waits on another, so there is
  * no device-side wait that could time out.  Steps are replayed from CUDA
  * graphs recorded on first use.  Each member's results are bit-identical to
  * stepping it alone with cmrt_step.
@@ -363,8 +363,8 @@ cmrt_status cmrt_batch_step(cmrt_batch* b, int64_t n);
  * state does not advance.  cache_path (may be NULL): a JSON array, one
  * object per line, keyed by device name, SM count and the batch signature
  * (revision of the batched kernel, precision, vector path, strip window,
- * size classes with their counts); a matching entry is applied without measuring unless flags has CMRT_TUNE_FORCE, and
- * a measurement replaces it.  us_per_step (may be NULL) receives the best
+ * size classes with their counts); a matching entry is applied without
+ * measuring unless flags has CMRT_TUNE_FORCE, and a measurement replaces it.  us_per_step (may be NULL) receives the best
  * time of one batched step in microseconds (the cached one on a hit). */
 cmrt_status cmrt_batch_tune(cmrt_batch* b, const char* cache_path, int32_t flags, double* us_per_step);
 

@@ -77,7 +77,9 @@ cudaError_t batch_launch(const BatchArgs& A, int grid, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// f(layout, vec, walls) with the march's layout for a batch's form
+// f(layout, vec, walls) with the march's layout for a batch's form.  (16-bit rows copied
+// 4 bytes at a time keep the periodic form here: without the tile in registers it does
+// not spill, as it does in the kernel of one lattice; FP32 with walls spills 4 bytes.)
 template <class F>
 cudaError_t with_layout(const BatchForm& b, F&& f) {
     using Yes = std::true_type;

@@ -173,7 +173,7 @@ __device__ __forceinline__ void segregation(float sx, float sy, float (&seg)[9])
     seg[7] = -d3;
 }
 
-// Reference dipoles of the 16-bit storage (cmrt_step.cu): per (red, blue)
+// Reference dipoles of the 16-bit storage (Layout16): per (red, blue)
 // pair, the velocity term of the equilibrium, 3 w_i rho_C c_i . u, plus the
 // segregation term of the recolour (Eq. eq_re_color), +/- w_i S . c-hat_i
 // (red +, blue -), for the links c = (1, 0) (D[0]), (0, 1) (D[1]), (1, 1)

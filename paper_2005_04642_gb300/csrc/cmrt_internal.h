@@ -1,5 +1,5 @@
-// Internal interface between the C ABI (cmrt_api.cu) and the kernels
-// (cmrt_step.cu, cmrt_aux.cu) of libcmrt.  Not installed, not part of the ABI.
+// Internal interface between the C ABI (cmrt_api.cu) and the kernels (the other
+// sources) of libcmrt.  Not installed, not part of the ABI.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -94,8 +94,8 @@ enum FwdPlane : int {
 
 // Geometry of the fused row-marching kernel: a CTA owns a strip of kTileX
 // columns (plus a 4-column halo on each side, kWin columns in all) and marches
-// down a segment of rows of it (chain_rows); each of its thread groups has
-// kThreads threads, one per window column.
+// down a segment of rows of it (chain_rows), with kThreads threads, one per window
+// column.
 constexpr int kThreads = 128;
 constexpr int kWin = 128;
 constexpr int kHalo = 4;
@@ -228,7 +228,7 @@ cudaError_t launch_adjoint_init(const float* pre0, const float* lam_pre0, const 
 cudaError_t launch_adjoint_reduce(const double* partials, int nblocks, double* out, cudaStream_t s);
 
 // 16-bit storage: FP32 post-collision planes float[18][ny][nx] <-> the
-// deviation layout of P.precision (see cmrt_step.cu).
+// record of P.precision (Layout16 in cmrt_march.cuh).
 cudaError_t launch_encode(const float* post32, const StepParams& P, void* state, cudaStream_t s);
 cudaError_t launch_decode(const void* state, const StepParams& P, float* post32, cudaStream_t s);
 

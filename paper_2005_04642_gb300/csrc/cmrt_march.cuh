@@ -91,10 +91,9 @@ __device__ __forceinline__ float2 sum9x2(const float (&r)[9], const float (&b)[9
 }
 
 // ---------------------------------------------------------------------------
-// Storage layouts.  A layout fixes the bytes of one ring row, how a thread
-// copies its share of a row from HBM, how stage A / D gather the 18
-// pre-collision populations of a node from the ring, and how stage D stores
-// the node's post-collision populations.
+// The 16-bit record: how a node is decoded, and encoded by the step's last stage.
+// (How the march copies rows of either storage and hands them to stage A: MarchF32
+// and March16.)
 // ---------------------------------------------------------------------------
 
 // 16-bit deviations (H = __half2 or __nv_bfloat162).
@@ -116,12 +115,6 @@ __device__ __forceinline__ float2 sum9x2(const float (&r)[9], const float (&b)[9
 // deviations.  The rest populations are the remainder of rho_C after the
 // decoded moving links, so that a record decodes to populations summing to
 // rho_C.  Any pair of population sets is representable.
-//
-// A ring row keeps, per window column, the densities as copied --
-// overwritten by the thread that copied them, as soon as its copy has landed
-// (prep), with the axis reference pair (rho_R psi^R_a, rho_B psi^B_a) -- the
-// diagonal reference pair (prep), and the rest populations and the twelve
-// 16-bit pairs as copied.
 template <class H>
 struct Layout16 {
     static constexpr int kPairPlanes = 12;  // four dipoles, eight deviations
@@ -239,7 +232,7 @@ struct Layout16 {
         const float2 mS = make_float2(-S, -S), pS = make_float2(S, S), m1 = make_float2(-1.0f, -1.0f);
         const float2 un2 = make_float2(P.dev_unscale, P.dev_unscale);
         // The rest populations are what is left of rho_R and rho_B after the
-        // moving links as the decoder will see them (pair(), bit for bit), so
+        // moving links as the decoder will see them (decode(), bit for bit), so
         // that every record decodes to exactly its colour densities: colour mass
         // is conserved through the storage to the rounding of that sum.
         float2 sum = make_float2(0.0f, 0.0f);
@@ -308,7 +301,8 @@ __device__ __forceinline__ float node_viscosity(float rr, float rb, float inv_rh
 //   warps stand on an SM: 512 columns in flight, against 256 with two CTAs of
 //   eight warps that split the stages between them, and each warp has the whole
 //   work of a row to overlap the others' barriers.
-// - Instructions per node fell from 836 to 600 (FP16: 1140 to 800).
+// - 630 thread instructions per node, 834 with FP16 storage (836 and 1140 where two
+//   groups of warps split the stages).
 // Measured at 8192^2 (drops, FP32): 1982 us per step before (33.9 GLUPS,
 // 4.9 TB/s), 1643 us now (40.9 GLUPS, 5.9 TB/s, 87 % of the measured copy);
 // 2048^2 143 -> 120 us; FP16 8192^2 2488 -> 1893 us, BF16 2614 -> 2001 us (bound
@@ -573,7 +567,8 @@ __device__ __forceinline__ void march_tile(char* __restrict__ smem, const Tile& 
 #pragma unroll
     for (int j = 0; j < L::kSlots - 1; ++j) issue(j);
 
-    // diagnostics: up to eight rows' sums, and the fastest node so far
+    // diagnostics: up to eight rows' sums, and the fastest node so far (the FP32 forms
+    // spill 16 to 28 bytes for them)
     Sum3 sum_mass, sum_mom;
     Fastest fastest;
     // what the later stages of this column need.  f, rho_R, rho_B and j: before an
@@ -866,9 +861,8 @@ __global__ void __launch_bounds__(L::W, march_ctas<L::W>())
 // 2x (H = 16) to 5x (H = 8) the arithmetic and L2 reads, which idle SMs have
 // to spare.  The arithmetic is the march's, expression by expression: both
 // give the same bits.
-// Measured per step (march -> this kernel; start of the change's tree in
-// brackets): 64^2 6.5 -> 2.05 us [5.2], 128^2 7.7 -> 2.75 [6.9], 256^2 10.3 ->
-// 4.2 [10.1], 1024 x 128 10.9 -> 7.2 [10.3], 512^2 21 -> 12.4 [22.9].
+// Measured per step, march -> this kernel: 64^2 6.5 -> 2.05 us, 128^2 7.7 -> 2.75,
+// 256^2 10.3 -> 4.2, 1024 x 128 10.9 -> 7.2, 512^2 21 -> 12.4.
 //
 // 16-bit storage: each thread first decodes its node's record into FP32
 // populations in shared memory (one more halo node and barrier: 24 x (H - 8)

@@ -949,7 +949,8 @@ __global__ void __launch_bounds__(kWin, 5) k_rev_tail(const StepParams P, const 
 //   window's own nodes are 24 x (H - 8).
 // - whole (tiny lattices, where launches count): the reverse collision too, its
 //   inputs loaded once and nothing but lambda written; 22 x (H - 10) own nodes,
-//   so that every collision runs 4 to 6 times.
+//   so that every collision runs 4 to 6 times.  With 16 window rows (64 registers) it
+//   spills 36 to 60 bytes, with 12 nothing.
 // The arithmetic is that of the plane passes, term by term in the same order.
 // VJP (cmrt_step_vjp): lam_out is the adjoint of f(t) (one halo node less), and
 // the whole form takes lam as the adjoint of f(t + 1), in the public layout.
@@ -1528,8 +1529,8 @@ __global__ void __launch_bounds__(kAT) k_init_T(const float* __restrict__ pre0, 
 // share of the rows (a warp reads four rows of eight slots at once), then the
 // first over the shares through distributed shared memory.  A fixed order, so
 // the sums are reproducible.  One CTA of 128 threads took 208 us for the 32768
-// rows of a 2048^2 lattice and 26 us for 3072, a load latency per 128 rows; this
-// takes 9 and 4 us.
+// rows of a 2048^2 lattice, a load latency per 128 rows; this takes 14 us (both
+// cold, under ncu).
 constexpr int kRedCtas = 8, kRedThreads = 512;
 __global__ void __cluster_dims__(kRedCtas, 1, 1) __launch_bounds__(kRedThreads)
     k_adj_reduce(const double* __restrict__ partials, int nblocks, double* __restrict__ out) {

@@ -51,12 +51,15 @@ dim3 chain_grid(int nx, int ny, int rows) {
 }
 
 int chain_rows(int nx, int ny, int sms, int precision) {
-    // Rows per CTA.  A CTA spends rows + 7 row iterations (7 fill the
-    // pipeline, 9 with 16-bit storage); an iteration takes longer the more CTAs
-    // share its SM: 0.79, 0.95, 1.40 and 1.47 us with one to four (FP32, states
-    // within L2).  Within one wave the fullest SM sets the time, by a quarter
-    // more where the state is beyond L2 (2048^2: 120 us with 64 rows in one wave,
-    // 129 with 32; 4096^2: 505 us with 241 rows, 435 with 64).  Past one wave the
+    // Rows per CTA.  A CTA spends rows + 7 row iterations (7 fill the pipeline; with
+    // 16-bit storage ten, of which three only decode and count as two: with a fill of
+    // ten FP16 4096 x 2048 takes 271 us instead of 265, 774 x 2786 113 instead of 105,
+    // 1308 x 623 36 instead of 33; 6902 x 648 196 instead of 201, BF16 4488 x 6270 847
+    // instead of 868); an iteration takes longer the more CTAs share its SM: 0.79,
+    // 0.95, 1.40 and 1.47 us with one to four (FP32, states within L2; 16-bit storage
+    // goes by the same ratios).  Within one wave the fullest SM sets the time, by a
+    // quarter more where the state is beyond L2 (2048^2: 120 us with 64 rows in one
+    // wave, 129 with 32; 4096^2: 505 us with 241 rows, 435 with 64).  Past one wave the
     // hardware hands out CTAs as others finish, which evens out the SMs'
     // different speeds (two dies), and half a CTA's time is lost at the end.
     // Measured at 8192^2: 36.3, 38.0, 40.4, 40.6, 40.9, 40.5 and 39.5 GLUPS with
