@@ -676,7 +676,7 @@ cmrt_status cmrt_fields(cmrt_ctx* h, float* rho_r, float* rho_b, float* ux, floa
     const size_t n = cells(*c);
     float* outs[5] = {rho_r, rho_b, ux, uy, p};
     float* dev[5];
-    bool any_host = false;
+    bool any_host = false, mapped = false;
     // device memory and mapped page-locked host memory are written by the
     // kernel in place; other host outputs go to the idle state buffer (5 of
     // its 11 or 18 floats per node) and are copied out
@@ -686,6 +686,7 @@ cmrt_status cmrt_fields(cmrt_ctx* h, float* rho_r, float* rho_b, float* ux, floa
         if (outs[k] && !is_device_ptr(outs[k])) {
             dev[k] = static_cast<float*>(mapped_host(c, outs[k]));
             copy[k] = !dev[k];
+            mapped = mapped || dev[k];
             any_host = true;
         }
     }
@@ -703,7 +704,7 @@ cmrt_status cmrt_fields(cmrt_ctx* h, float* rho_r, float* rho_b, float* ux, floa
     if (c->p.stencil_order == 6) {
         CK(c, cmrt::launch_fields6(static_cast<const float*>(c->buf[c->cur]), c->sp, fo, c->stream));
     } else {
-        CK(c, cmrt::launch_fields(c->buf[c->cur], c->sp, c->rows, fo, c->stream));
+        CK(c, cmrt::launch_fields(c->buf[c->cur], c->sp, c->rows, fo, mapped, c->stream));
     }
     c->launches++;
     if (any_host) {

@@ -133,8 +133,9 @@ cudaError_t launch_diag_partials16(const void* src, const StepParams& P, int row
 // The forward fields alone (lattices the small-lattice kernel takes, FP32
 // storage), the same bits as launch_step_fields.
 cudaError_t launch_fwd_fields(const float* src, const StepParams& P, float* fwd, cudaStream_t s);
-// Fields of the state whose post-collision populations are in src.
-cudaError_t launch_fields(const void* src, const StepParams& P, int rows, FieldOut out, cudaStream_t s);
+// Fields of the state whose post-collision populations are in src; host: into
+// page-locked host memory (some of them).
+cudaError_t launch_fields(const void* src, const StepParams& P, int rows, FieldOut out, bool host, cudaStream_t s);
 // Per-CTA FP64 partial diagnostics into partials[grid][kDiagSlots].
 cudaError_t launch_diag_partials(const void* src, const StepParams& P, int rows, double* partials, cudaStream_t s);
 // Same, from pre-collision FP32 populations in the public layout float[2][9][ny][nx].

@@ -106,13 +106,18 @@ cudaError_t launch_fwd_fields(const float* src, const StepParams& P, float* fwd,
     return launch_small_any<MarchF32<kWin>, Pass::FwdFields>(src, nullptr, P, fo, nullptr, s);
 }
 
-cudaError_t launch_fields(const void* src, const StepParams& P, int rows, FieldOut out, cudaStream_t s) {
+cudaError_t launch_fields(const void* src, const StepParams& P, int rows, FieldOut out, bool host, cudaStream_t s) {
+    // Page-locked outputs of an odd width: strips share 32-byte sectors, which fewer, longer
+    // segments write closer together in time.  4095 x 1024 651 -> 609 us (581 before the
+    // march), 701^2 87 -> 82 (80), FP16 4095 x 1024 660 -> 596 (593); not small lattices
+    // (FP16 701^2 85 -> 94)
+    if (host && P.nx % 4 != 0 && static_cast<long>(P.nx) * P.ny > (P.precision == kPrecF32 ? 400000 : 600000)) rows *= 4;
     if (P.precision != kPrecF32) return launch_fields16(src, P, rows, out, s);
     // 4-byte copies (nx no multiple of 4) in one wave of long segments: half the rows, in
     // two waves, even out the SMs.  4095 x 1024 148 -> 128 us, 3001 x 2000 204 -> 173;
     // not segments of 32 rows (1501 x 1500 77 -> 80) or several waves (6001 x 3001 473 -> 499)
     const dim3 g = chain_grid(P.nx, P.ny, rows);
-    if (P.nx % 4 != 0 && rows > 48 && static_cast<long>(g.x) * g.y <= 4 * 152) rows /= 2;
+    if (!host && P.nx % 4 != 0 && rows > 48 && static_cast<long>(g.x) * g.y <= 4 * 152) rows /= 2;
     return launch_march<MarchF32<kWin>, Pass::Fields>(src, nullptr, P, rows, out, nullptr, nullptr, s);
 }
 
